@@ -45,7 +45,7 @@ extern "C" {
 #define AFC_FP32_RECHECK 1  /* delta in FP32, realizations with a near-tied top two in FP64 */
 
 #define AFC_PATH_AUTO 0     /* counting path chosen by what fits in shared memory            */
-                            /* (a CTA must hold at least six source slots)                   */
+                            /* (a CTA must hold at least eight source slots)                 */
 #define AFC_PATH_SHARED 1   /* realization and source state in shared memory (small graphs)  */
 #define AFC_PATH_GLOBAL 2   /* realized graph and source state in device memory (any size)   */
 
@@ -111,7 +111,7 @@ typedef struct {
   int32_t slots_per_team;    /* sources a team advances in lockstep (1..16); 0 = as many   */
                              /* as shared memory holds                                     */
   int32_t memory_path;       /* AFC_PATH_AUTO: realizations of graphs whose CTA holds the  */
-                             /* realization and at least six source slots in shared memory */
+                             /* realization and at least eight source slots in shared memory */
                              /* run there, others on the global-memory path;               */
                              /* AFC_PATH_SHARED / AFC_PATH_GLOBAL force one                 */
                              /* (AFC_EUNSUPPORTED if the shared path does not fit)          */

@@ -129,6 +129,26 @@ int validate(const afc_mc_problem *p) {
   return AFC_OK;
 }
 
+// The LONG form of the settle-step routine (StepGraph in mc_steps.cuh): its extra bookkeeping pays
+// with long lengths; with short ones the settle steps are about the levels already.  Measured on
+// the shared path (n = 1,000, ms a call of 1,200 realizations, LONG / plain): ER lengths 1..20
+// 111 / 107, 1..30 116 / 119, 1..50 124 / 137; WS 1..10 86 / 89, 1..20 96 / 110.  On the global
+// path, where the arena's latency hides part of the steps, ER n = 3,000 (107 realizations) 1..50
+// 200 / 188, 1..100 218 / 226; WS 1..50 178 / 180, 1..100 190 / 210.  A per-edge array of largest
+// lengths is not known here: the plain form takes any.
+constexpr uint32_t kLongLen = 24, kLongLenGlobal = 64;
+bool fits_long(const afc_mc_problem &p) {
+  return !p.w_hi && p.w_hi_all <= 32767u && (uint64_t)p.n * p.w_hi_all < (1ull << 30);
+}
+// The r-hop neighbourhoods of the row-wise mode are too small to win back the LONG tables (76 nodes,
+// 1-hop balls: 0.89 against 0.82 ms a call).
+bool prefers_long(const afc_mc_problem &p) {
+  return fits_long(p) && p.w_hi_all >= kLongLen && !(p.per_row && p.hop_radius);
+}
+bool prefers_long_global(const afc_mc_problem &p) {
+  return fits_long(p) && p.w_hi_all >= kLongLenGlobal;
+}
+
 McDev to_dev(const afc_mc_problem &p, uint32_t r_begin, uint32_t *counts, afc_mc_stats *stats,
              double *dump_bc, int32_t *dump_next) {
   McDev d{};
@@ -253,7 +273,7 @@ BigPlan plan_big(const afc_mc_problem &p, uint64_t r_count) {
   BigPlan b;
   const uint32_t n = (uint32_t)p.n;
   const uint64_t arcs = 2ull * (uint64_t)p.m;
-  const uint32_t per_warp = (4u * n + 15u) & ~15u;   // one distance array
+  const uint32_t per_warp = big_step_smem_bytes(n, prefers_long_global(p));
   const uint32_t fit = (uint32_t)std::max(0, d.smem_optin - 1024) / per_warp;
   if (p.team_threads == 0 && fit >= kMinStepWarps && steps_beat_buckets(p)) {
     // settle-step kernel: one source per warp, its distances on chip (16 warps per CTA at most:
@@ -263,7 +283,7 @@ BigPlan plan_big(const afc_mc_problem &p, uint64_t r_count) {
     b.spt = std::min<uint32_t>(fit, (uint32_t)b.block / 32u);
     b.on_chip = 1;
     if (!p.block_threads && b.spt <= 8) b.block = 256;
-    b.smem = b.on_chip ? b.spt * per_warp : 0u;
+    b.smem = b.spt * per_warp;
     b.slot_stride = big_step_slot_bytes(n, !b.on_chip);
     const uint32_t per_sm = std::max<uint32_t>(
         1u, std::min<uint32_t>(2048u / (uint32_t)b.block, (228u * 1024u) / (b.smem + 1024u)));
@@ -359,10 +379,11 @@ bool smem_fits(const afc_mc_problem &p) {
 }
 
 // AFC_PATH_AUTO: the shared-memory path when shared memory holds at least this many compact
-// source slots.  Measured on mix graphs (mean degree 8, FP64): with 7 slots (1,771 nodes) it
-// is 7% faster than the global path's settle-step kernel, with 6 slots (2,014 nodes) 3%
-// faster, with 5 slots (2,161-2,340 nodes) 7-8% slower.
-constexpr uint32_t kMinSharedSlots = 6;
+// source slots.  Measured on graphs of mean degree 8 (ms a call, shared / global settle-step
+// kernel; WS lengths 1..50, ER 1..10 in FP32, ER 1..100): 8 slots (n = 1,592, 431 realizations)
+// 192 / 202, 106 / 134, 218 / 213; 7 slots (n = 1,700, 373) 217 / 197, 165 / 132, 249 / 209; 6
+// slots (n = 2,000, 261) 259 / 189, 138 / 127, 301 / 205.
+constexpr uint32_t kMinSharedSlots = 8;
 
 bool wants_global(const afc_mc_problem &p) {
   if (p.memory_path == AFC_PATH_GLOBAL) return true;
@@ -383,6 +404,7 @@ struct SharedBatch {
   uint32_t nmax = 1;
   uint64_t amax = 1, items = 0;
   uint32_t want_warps = 0;
+  bool long_form = false;   // the source routine's form: by most of the batch's work
   McPlan pl;
   size_t scratch_stride = 0, scratch_bytes = 0;
 };
@@ -394,15 +416,28 @@ SharedBatch shared_batch(int nprob, const afc_mc_problem *probs, const uint32_t 
   if (sb.order.empty()) return sb;
   const DevInfo di = dev_info();
   const uint32_t cap = (uint32_t)std::max(0, di.smem_optin - 1024);
+  double work = 0.0, small_work = 0.0, long_work = 0.0;
+  bool may_long = true;
   for (int g : sb.order) {
     const afc_mc_problem &p = probs[g];
     sb.nmax = std::max<uint32_t>(sb.nmax, (uint32_t)p.n);
     sb.amax = std::max<uint64_t>(sb.amax, 2ull * (uint64_t)p.m);
     // no count given: size for a launch that fills the GPU
     sb.items += r_count ? items_of(p, r_count[g]) : (uint64_t)1 << 40;
-    if (sb.order.size() > 1)
-      sb.want_warps = std::max(sb.want_warps, slots_within((uint32_t)p.n, 2ull * (uint64_t)p.m, cap));
+    const uint32_t slots = slots_within((uint32_t)p.n, 2ull * (uint64_t)p.m, cap);
+    const double per = (double)p.n * (double)(p.n + 2 * p.m) * (r_count ? (double)items_of(p, r_count[g]) : 1.0);
+    work += per;
+    if (slots > 16u) small_work += per;
+    if (prefers_long(p)) long_work += per;
+    may_long = may_long && fits_long(p);
+    if (sb.order.size() > 1) sb.want_warps = std::max(sb.want_warps, slots);
   }
+  // A batch's CTAs have 1024 threads only when the graphs that can use more than 16 source warps
+  // (about n < 950) are most of its work: at 512 threads the source warps of the others keep up
+  // to 128 registers instead of 64 (8 graphs of 230-1,730 nodes, 96 realizations each: 138 ms a
+  // call with 1024 threads, 124 ms with 512).
+  sb.long_form = may_long && long_work > 0.5 * work;
+  if (small_work <= 0.5 * work) sb.want_warps = std::min(sb.want_warps, 16u);
   sb.pl = plan_for(probs[sb.order[0]], sb.nmax, sb.amax, std::max<uint64_t>(sb.items, 1),
                    sb.want_warps);
   sb.scratch_stride = (mc_cta_scratch_bytes(sb.nmax) + 255) & ~size_t(255);
@@ -481,7 +516,7 @@ int run_counts(int nprob, const afc_mc_problem *probs, const uint32_t *r_begin,
     }
     // the shared batch's grid was sized for all its items: the launch may use fewer CTAs
     const uint32_t grid = (uint32_t)std::min<uint64_t>(pl.grid, prefix[ns]);
-    cudaError_t e = launch_mc_counts(pl.block, devs_d, ns, prefix_d, prefix[ns], pl.nsw, pl.smem,
+    cudaError_t e = launch_mc_counts(pl.block, sb.long_form, devs_d, ns, prefix_d, prefix[ns], pl.nsw, pl.smem,
                                      std::max<uint32_t>(grid, 1u), ws + meta_bytes(nprob),
                                      sb.scratch_stride, stream);
     if (e != cudaSuccess) return cuda_fail(e, "counting kernel launch");
@@ -499,7 +534,7 @@ int run_counts(int nprob, const afc_mc_problem *probs, const uint32_t *r_begin,
     BigGroup *groups_d = reinterpret_cast<BigGroup *>(bigbase + b.off_groups);
     AFC_CUDA(cudaMemcpyAsync(groups_d, groups.data(), sizeof(BigGroup) * b.ngroups,
                              cudaMemcpyHostToDevice, stream));
-    cudaError_t e = launch_mc_global(b.block, b.team, devs_d + k, p.precision, groups_d, b.ngroups,
+    cudaError_t e = launch_mc_global(b.block, b.team, prefers_long_global(p), devs_d + k, p.precision, groups_d, b.ngroups,
                                      rc, bigbase + b.off_arena, b.slot_stride, b.spt, b.smem, b.on_chip,
                                      b.grid, stream);
     if (e != cudaSuccess) return cuda_fail(e, "global-path counting launch");
@@ -776,7 +811,7 @@ int afc_debug_sssp(const afc_mc_problem *prob, uint32_t r, const int32_t *source
   const McPlan pl = plan_for(*prob, (uint32_t)prob->n, 2ull * (uint64_t)prob->m, (uint64_t)nsrc);
   if (!pl.fits) return fail(AFC_EUNSUPPORTED, "graph too large for the shared-memory SSSP kernel");
   McDev d = to_dev(*prob, 0, nullptr, stats, nullptr, nullptr);
-  cudaError_t e = launch_debug_sssp(pl.block, d, r, sources, nsrc, pl.nsw, pl.smem, dist, sigma,
+  cudaError_t e = launch_debug_sssp(pl.block, d, r, sources, nsrc, pl.nsw, prefers_long(*prob), pl.smem, dist, sigma,
                                     (cudaStream_t)stream);
   return e == cudaSuccess ? AFC_OK : cuda_fail(e, "debug_sssp");
 }

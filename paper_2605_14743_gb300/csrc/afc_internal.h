@@ -15,6 +15,7 @@ size_t big_group_bytes(uint32_t n, uint64_t arcs);
 uint32_t big_slot_bytes(uint32_t n);
 // bytes of one warp's region of the arena on the settle-step global path (path counts, settle
 // order, pending list, and the distances when they are not kept on chip)
+uint32_t big_step_smem_bytes(uint32_t n, bool long_form);
 size_t big_step_slot_bytes(uint32_t n, bool dist_in_arena);
 void big_group_carve(BigGroup &G, unsigned char *base, uint32_t n, uint64_t arcs);
 bool big_config_supported(int block, int team);
@@ -27,7 +28,7 @@ bool big_config_supported(int block, int team);
 uint32_t big_dist_smem_bytes(uint32_t n, uint32_t nslots);
 // Shared memory of a Brandes CTA that keeps its whole slots (stride big_slot_bytes) on chip.
 uint32_t big_slots_smem_bytes(uint32_t n, uint32_t nslots);
-cudaError_t launch_mc_global(int block, int team, const McDev *Pd, int precision,
+cudaError_t launch_mc_global(int block, int team, bool long_form, const McDev *Pd, int precision,
                              BigGroup *groups_d, uint32_t ngroups, uint32_t r_count,
                              unsigned char *arena, size_t slot_stride, uint32_t spt,
                              uint32_t smem_bytes, int slots_on_chip, uint32_t grid,
@@ -58,7 +59,8 @@ uint32_t mc_slots_within(uint32_t n, uint64_t arcs, uint32_t bytes);
 // Device memory of one counting CTA of the shared-memory path (graphs of up to n nodes):
 // components, source list, selection scratch and betweenness accumulators.
 size_t mc_cta_scratch_bytes(uint32_t n);
-cudaError_t launch_mc_counts(int block, const McDev *probs_dev, int nprob,
+// long_form: the LONG form of the source routine (StepGraph in mc_steps.cuh)
+cudaError_t launch_mc_counts(int block, bool long_form, const McDev *probs_dev, int nprob,
                              const uint64_t *prefix_dev, uint64_t total_items,
                              uint32_t source_warps, uint32_t smem_bytes, uint32_t grid,
                              unsigned char *scratch, size_t scratch_stride, cudaStream_t stream);
@@ -67,7 +69,7 @@ cudaError_t launch_debug_realize(const McDev &P, uint32_t r_count, uint8_t *aliv
 cudaError_t launch_debug_components(const McDev &P, uint32_t r_count, int32_t *comp,
                                     int32_t *csize, cudaStream_t stream);
 cudaError_t launch_debug_sssp(int block, const McDev &P, uint32_t r, const int32_t *sources,
-                              int32_t nsrc, uint32_t source_warps, uint32_t smem, uint32_t *dist,
+                              int32_t nsrc, uint32_t source_warps, bool long_form, uint32_t smem, uint32_t *dist,
                               uint64_t *sigma, cudaStream_t stream);
 
 // solve.cu / perturb.cu

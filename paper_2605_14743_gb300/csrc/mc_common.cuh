@@ -225,34 +225,33 @@ struct BcAcc {
   unsigned long long *a0, *a1, *a2;
 };
 
-// Betweenness accumulation without return values (device-memory reductions): the addend x
-// (0 <= x < 2^64) is split exactly, from its bits, into x 2^64 = xi 2^64 + xf (xf < 2^64,
-// truncated below 2^-64, i.e. exact whenever x >= 2^-12), and xi, the top and the bottom 32 bits of xf go to three
-// 64-bit sums (each far from overflow for fewer than 2^31 addends).  Integer additions are
-// associative, so the total is exact and independent of the order.
+// Betweenness accumulation without return values (device-memory reductions): a dependency x
+// (0 <= x < 2^16: it is at most the number of other nodes) is split exactly, from its bits, into
+// x 2^64 = xi 2^64 + xf (xf < 2^64, truncated below 2^-64, i.e. exact whenever x >= 2^-12), and xi,
+// the top and the bottom 32 bits of xf go to three 64-bit sums (each far from overflow for fewer
+// than 2^31 addends).  Integer additions are associative, so the total is exact and independent
+// of the order.  The split takes 32-bit funnel shifts: with x below 2^20 the shifts of its 53-bit
+// significand stay below 32 places to the left.
 __device__ __forceinline__ void fx_red(unsigned long long *a0, unsigned long long *a1,
                                        unsigned long long *a2, uint32_t v, double x) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const int ex = (int)((b >> 52) & 0x7FFu);
-  if (ex == 0 || (b >> 63)) return;
-  const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-  const int sh = ex - 1075 + 64;
-  unsigned long long xi, xf;
-  if (sh >= 64) {
-    xi = m << (sh - 64);
-    xf = 0ull;
-  } else if (sh > 0) {
-    xi = m >> (64 - sh);
-    xf = m << sh;
-  } else if (sh > -53) {
-    xi = 0ull;
-    xf = m >> (-sh);
+  const uint32_t top = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const int ex = (int)(top >> 20);   // sign 0
+  if (ex == 0 || ex > 1023 + 20) return;
+  const uint32_t hi = (top & 0xFFFFFu) | 0x100000u;
+  const int sh = ex - 1011;   // x 2^64 = (hi:lo) << sh
+  uint32_t xi = 0u, f1, f0;
+  if (sh > 0) {               // 1 .. 32
+    xi = __funnelshift_lc(hi, 0u, (uint32_t)sh);
+    f1 = __funnelshift_lc(lo, hi, (uint32_t)sh);
+    f0 = __funnelshift_lc(0u, lo, (uint32_t)sh);
   } else {
-    return;
+    const uint32_t k = (uint32_t)-sh;
+    f1 = k < 32u ? hi >> k : 0u;
+    f0 = k < 32u ? __funnelshift_r(lo, hi, k) : k < 64u ? hi >> (k - 32u) : 0u;
   }
-  if (xi) atomicAdd(&a0[v], xi);
-  if (xf >> 32) atomicAdd(&a1[v], xf >> 32);
-  if (xf & 0xFFFFFFFFull) atomicAdd(&a2[v], xf & 0xFFFFFFFFull);
+  if (xi) atomicAdd(&a0[v], (unsigned long long)xi);
+  if (f1) atomicAdd(&a1[v], (unsigned long long)f1);
+  if (f0) atomicAdd(&a2[v], (unsigned long long)f0);
 }
 
 // B_v as a double, written over a0 (each thread converts its own entries).
@@ -272,9 +271,9 @@ __device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
 
 // The dependency step of v from acc = sum of its successors' rho (Sec. 3.1, Brandes):
 // delta(v) = sigma(v) acc and rho(v) = (1 + delta(v)) / sigma(v) = acc + 1 / sigma(v).
-template <typename DT>
-__device__ __forceinline__ void dependency(uint64_t sg, DT acc, DT &dep, DT &rho) {
-  if (sg == 1ull) {
+template <typename DT, typename SG>
+__device__ __forceinline__ void dependency(SG sg, DT acc, DT &dep, DT &rho) {
+  if (sg == (SG)1) {
     dep = acc;
     rho = (DT)1 + dep;
   } else {
@@ -691,7 +690,7 @@ __device__ __forceinline__ bool brandes_batch(const Team<TS, BLOCK> &team, const
               if (!is_src && acc_i) atomicAdd(&acc.a0[v], (unsigned long long)acc_i);
             } else {
               DT dep, rho;
-              dependency<DT>(sg, (DT)acc_i + acc_f, dep, rho);
+              dependency<DT, uint64_t>(sg, (DT)acc_i + acc_f, dep, rho);
               uint64_t bits = 0;
               *reinterpret_cast<DT *>(&bits) = rho;
               a.sig[v] = bits;

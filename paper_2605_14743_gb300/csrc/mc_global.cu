@@ -22,12 +22,20 @@ namespace afc {
 
 __host__ __device__ inline size_t al256(size_t x) { return (x + 255u) & ~size_t(255); }
 
+// Shared memory of one source warp of the settle-step kernel: its distance array where it fits
+// and, for the LONG form, its level counters (few: what shared memory takes, L1 lacks).
+__host__ __device__ inline uint32_t big_step_chip_bytes(uint32_t n, bool dist_on_chip,
+                                                        bool long_form) {
+  return (long_form ? 4u * kLevelHist : 0u) + (dist_on_chip ? al16(4u * n) : 0u);
+}
+
 namespace {
 
 constexpr int kPrepThreads = 1024;
 
 __global__ void __launch_bounds__(kPrepThreads, 1)
-big_prep_kernel(const McDev *__restrict__ Pd, BigGroup *groups, uint32_t r0, uint32_t r_count) {
+big_prep_kernel(const McDev *__restrict__ Pd, BigGroup *groups, uint32_t r0, uint32_t r_count,
+                int steps, int long_form) {
   extern __shared__ __align__(16) unsigned char smem[];
   CtaCtl *ctl = reinterpret_cast<CtaCtl *>(smem);
   const McDev &P = *Pd;
@@ -51,7 +59,12 @@ big_prep_kernel(const McDev *__restrict__ Pd, BigGroup *groups, uint32_t r0, uin
   components(P, H, G.comp, G.cinfo);
   if (P.per_row) keep_anchor_component(n, anchor, G.comp, G.cinfo);
   bucket_setup(ctl, P.delta);
-  min_lengths(H, G.mw);
+  // the settle-step kernel's tables; the bucketed kernel reads the plain arcs
+  if (steps) {
+    // lengths beyond the problem's declared largest one (the launch chose the form by it)
+    if (long_form && !long_lengths(n, ctl->wmax) && threadIdx.x == 0) ctl->err |= kErrInput;
+    step_tables(H, G.arc, G.mwt, long_form != 0);
+  }
   uint32_t *cedges = G.centre;   // scratch until selection
   for (uint32_t v = threadIdx.x; v < n; v += blockDim.x) {
     cedges[v] = 0; reinterpret_cast<unsigned long long *>(G.bc)[v] = 0ull;
@@ -93,6 +106,7 @@ big_prep_kernel(const McDev *__restrict__ Pd, BigGroup *groups, uint32_t r0, uin
     G.nsrc = ctl->nsrc;
     G.cursor = 0;
     G.dsh = ctl->dsh;
+    G.dbits = dist_bits(n, ctl->wmax) + (long_form ? 1u : 0u);
     G.err = ctl->err;
     G.ovf = 0;
     G.redo = 0;
@@ -156,7 +170,7 @@ big_brandes_kernel(const McDev *__restrict__ Pd, BigGroup *groups, uint32_t ngro
 // pending list in the warp's region of the device arena -- and claim the sources of the
 // groups one at a time, group by group, so the realized graph being worked on stays hot in L2.
 // mode as for big_brandes_kernel.
-template <int BLOCK>
+template <int BLOCK, bool LONG>
 __global__ void __launch_bounds__(BLOCK, 1)
 big_steps_kernel(const McDev *__restrict__ Pd, BigGroup *groups, uint32_t ngroups,
                  unsigned char *arena, size_t slot_stride, uint32_t nsw, int mode,
@@ -173,14 +187,15 @@ big_steps_kernel(const McDev *__restrict__ Pd, BigGroup *groups, uint32_t ngroup
   mine += al256(2ull * n);
   sl.plist = reinterpret_cast<uint16_t *>(mine);
   mine += al256(2ull * n);
-  sl.dist = dist_on_chip ? reinterpret_cast<uint32_t *>(smem + (size_t)warp * al16(4u * n))
-                         : reinterpret_cast<uint32_t *>(mine);
+  const uint32_t chip = big_step_chip_bytes(n, dist_on_chip != 0, LONG);   // per warp
+  sl.hist = reinterpret_cast<uint32_t *>(smem + (size_t)warp * chip);
+  sl.dist = dist_on_chip ? sl.hist + (LONG ? kLevelHist : 0u) : reinterpret_cast<uint32_t *>(mine);
   for (uint32_t g = 0; g < ngroups; ++g) {
     BigGroup &G = groups[g];
     if (!G.active || (mode == 2 && !G.redo)) continue;
-    const Realized H{n, G.rp, G.arc};
+    const StepGraph<uint32_t> H{n, G.rp, G.arc, G.mwt};
     const BcAcc acc{reinterpret_cast<unsigned long long *>(G.bc), G.a1, G.a2};
-    const uint32_t nsrc = G.nsrc;
+    const uint32_t nsrc = G.nsrc, dbits = G.dbits;
     uint32_t err = 0, ovf = 0;
     for (;;) {
       uint32_t k = 0;
@@ -188,10 +203,10 @@ big_steps_kernel(const McDev *__restrict__ Pd, BigGroup *groups, uint32_t ngroup
       k = __shfl_sync(kFull, k, 0);
       if (k >= nsrc) break;
       const uint32_t s = G.src[k];
-      const bool ok =
-          mode == 1 ? source_steps<float, false, false>(H, G.mw, sl, s, true, acc, err, ovf)
-                    : source_steps<double, false, false>(H, G.mw, sl, s, true, acc, err, ovf);
-      if (!ok) break;
+      const StepResult res =
+          mode == 1 ? source_steps<float, false, false, LONG>(H, sl, s, dbits, true, acc, err, ovf)
+                    : source_steps<double, false, false, LONG>(H, sl, s, dbits, true, acc, err, ovf);
+      if (res != StepResult::done) break;
     }
     err = __reduce_or_sync(kFull, err);
     ovf = __reduce_or_sync(kFull, ovf);
@@ -264,15 +279,15 @@ cudaError_t launch_brandes_t(const McDev *Pd, BigGroup *groups, uint32_t ngroups
   X(256, 64) X(256, 128) X(256, 256) X(512, 128) X(512, 256) X(512, 512) \
   X(1024, 128) X(1024, 256) X(1024, 512) X(1024, 1024)
 
-template <int BLOCK>
+template <int BLOCK, bool LONG>
 cudaError_t launch_steps_t(const McDev *Pd, BigGroup *groups, uint32_t ngroups,
                            unsigned char *arena, size_t stride, uint32_t nsw, int mode,
                            uint32_t smem_bytes, int dist_on_chip, uint32_t grid,
                            cudaStream_t stream) {
   if (smem_bytes > 48u * 1024u)
-    cudaFuncSetAttribute(big_steps_kernel<BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(big_steps_kernel<BLOCK, LONG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          smem_bytes);
-  big_steps_kernel<BLOCK><<<grid, BLOCK, smem_bytes, stream>>>(Pd, groups, ngroups, arena, stride,
+  big_steps_kernel<BLOCK, LONG><<<grid, BLOCK, smem_bytes, stream>>>(Pd, groups, ngroups, arena, stride,
                                                                nsw, mode, dist_on_chip);
   return cudaGetLastError();
 }
@@ -280,18 +295,18 @@ cudaError_t launch_steps_t(const McDev *Pd, BigGroup *groups, uint32_t ngroups,
 // team 0: the settle-step kernel with spt source warps per CTA (slots_on_chip: their distance
 // arrays in shared memory) in CTAs of 256 or 512 threads (1024 would cap the registers below
 // what the routine needs); otherwise the bucketed kernel with teams of `team` threads
-cudaError_t launch_brandes(int block, int team, const McDev *Pd, BigGroup *groups,
+cudaError_t launch_brandes(int block, int team, bool long_form, const McDev *Pd, BigGroup *groups,
                            uint32_t ngroups, unsigned char *arena, size_t stride, uint32_t spt,
                            int mode, uint32_t smem_bytes, int slots_on_chip, uint32_t grid,
                            cudaStream_t stream) {
   if (team == 0) {
     if (spt < 1 || spt > (uint32_t)block / 32u) return cudaErrorInvalidValue;
-    if (block == 256)
-      return launch_steps_t<256>(Pd, groups, ngroups, arena, stride, spt, mode, smem_bytes,
+#define AFC_X(B, LG)                                                                          \
+  if (block == B && long_form == LG)                                                          \
+    return launch_steps_t<B, LG>(Pd, groups, ngroups, arena, stride, spt, mode, smem_bytes,   \
                                  slots_on_chip, grid, stream);
-    if (block == 512)
-      return launch_steps_t<512>(Pd, groups, ngroups, arena, stride, spt, mode, smem_bytes,
-                                 slots_on_chip, grid, stream);
+    AFC_X(256, true) AFC_X(256, false) AFC_X(512, true) AFC_X(512, false)
+#undef AFC_X
     return cudaErrorInvalidValue;
   }
 #define AFC_X(B, T)                                                                   \
@@ -314,11 +329,15 @@ bool big_config_supported(int block, int team) {
 
 
 size_t big_group_bytes(uint32_t n, uint64_t arcs) {
-  return al256(4ull * (n + 1)) + al256(4ull * (arcs > 0 ? arcs : 1)) + 4 * al256(4ull * n) +
-         2 * al256(2ull * n) + 4 * al256(8ull * n);
+  return al256(4ull * (n + 1)) + al256(4ull * (arcs > 0 ? arcs : 1)) + 5 * al256(4ull * n) +
+         al256(2ull * n) + 4 * al256(8ull * n);
 }
 
 uint32_t big_slot_bytes(uint32_t n) { return (slot_bytes_for(n) + 255u) & ~255u; }
+
+uint32_t big_step_smem_bytes(uint32_t n, bool long_form) {
+  return big_step_chip_bytes(n, true, long_form);
+}
 
 size_t big_step_slot_bytes(uint32_t n, bool dist_in_arena) {
   return al256(8ull * n) + 2 * al256(2ull * n) + (dist_in_arena ? al256(4ull * n) : 0);
@@ -338,7 +357,7 @@ void big_group_carve(BigGroup &G, unsigned char *base, uint32_t n, uint64_t arcs
   G.bc = reinterpret_cast<double *>(take(8ull * n));
   G.a1 = reinterpret_cast<unsigned long long *>(take(8ull * n));
   G.a2 = reinterpret_cast<unsigned long long *>(take(8ull * n));
-  G.mw = reinterpret_cast<uint16_t *>(take(2ull * n));
+  G.mwt = reinterpret_cast<uint32_t *>(take(4ull * n));
   G.best = reinterpret_cast<unsigned long long *>(take(8ull * n));
 }
 
@@ -350,7 +369,7 @@ uint32_t big_slots_smem_bytes(uint32_t n, uint32_t nslots) {
   return al16((uint32_t)sizeof(CtaCtl)) + nslots * big_slot_bytes(n);
 }
 
-cudaError_t launch_mc_global(int block, int team, const McDev *Pd, int precision,
+cudaError_t launch_mc_global(int block, int team, bool long_form, const McDev *Pd, int precision,
                              BigGroup *groups_d, uint32_t ngroups, uint32_t r_count,
                              unsigned char *arena, size_t slot_stride, uint32_t spt,
                              uint32_t smem_bytes, int slots_on_chip, uint32_t grid,
@@ -358,16 +377,18 @@ cudaError_t launch_mc_global(int block, int team, const McDev *Pd, int precision
   if (team != 0 && !big_config_supported(block, team)) return cudaErrorInvalidValue;
   const bool fp32 = (precision == 1);
   for (uint32_t r0 = 0; r0 < r_count; r0 += ngroups) {
-    big_prep_kernel<<<ngroups, kPrepThreads, sizeof(CtaCtl), stream>>>(Pd, groups_d, r0, r_count);
+    big_prep_kernel<<<ngroups, kPrepThreads, sizeof(CtaCtl), stream>>>(Pd, groups_d, r0, r_count,
+                                                                           team == 0 ? 1 : 0,
+                                                                           long_form ? 1 : 0);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    e = launch_brandes(block, team, Pd, groups_d, ngroups, arena, slot_stride, spt, fp32 ? 1 : 0,
+    e = launch_brandes(block, team, long_form, Pd, groups_d, ngroups, arena, slot_stride, spt, fp32 ? 1 : 0,
                        smem_bytes, slots_on_chip, grid, stream);
     if (e != cudaSuccess) return e;
     big_select_kernel<<<ngroups, kPrepThreads, sizeof(CtaCtl), stream>>>(Pd, groups_d, fp32 ? 1 : 0, 0);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (fp32) {
-      e = launch_brandes(block, team, Pd, groups_d, ngroups, arena, slot_stride, spt, 2,
+      e = launch_brandes(block, team, long_form, Pd, groups_d, ngroups, arena, slot_stride, spt, 2,
                          smem_bytes, slots_on_chip, grid, stream);
       if (e != cudaSuccess) return e;
       big_select_kernel<<<ngroups, kPrepThreads, sizeof(CtaCtl), stream>>>(Pd, groups_d, 0, 1);

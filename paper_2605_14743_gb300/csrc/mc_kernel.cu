@@ -21,8 +21,9 @@
 
 namespace afc {
 
-// Shared-memory layout of a counting CTA: control head, the realization (rp, arcs, smallest
-// incident length) and the source slots.  What the source warps do not touch while they run
+// Shared-memory layout of a counting CTA: control head, the realization (16-bit row offsets,
+// arcs, per-node length bounds) and the source slots (whose bytes hold the 32-bit row offsets
+// while the realization is built).  What the source warps do not touch while they run
 // (components, the source list, selection scratch, betweenness accumulators) lives in the
 // CTA's region of device memory (CtaScratch), so that more source slots fit on chip.  The slot
 // region holds nsw compact slots (12 bytes per node, see StepSlot) and, reusing the same bytes,
@@ -34,9 +35,9 @@ struct StepLayout {
   __host__ __device__ static uint32_t al(uint32_t x) { return al16(x); }
   __host__ __device__ void make(uint32_t n, uint32_t arcs, uint32_t nsw) {
     uint32_t o = al(sizeof(CtaHead));
-    off_rp = o;     o = al(o + 4u * (n + 1));
+    off_rp = o;     o = al(o + 2u * (n + 1));
     off_arc = o;    o = al(o + 4u * (arcs > 0 ? arcs : 1));
-    off_mw = o;     o = al(o + 2u * n);
+    off_mw = o;     o = al(o + 4u * n);
     off_slots = o;
     slot_bytes = al(4u * n) + al(8u * n);
     wide_bytes = slot_bytes + 2u * al(2u * n);
@@ -55,6 +56,7 @@ struct StepLayout {
     s.sig = reinterpret_cast<uint64_t *>(p);   p += al(8u * n);
     s.ord = wide ? reinterpret_cast<uint16_t *>(p) : nullptr;   p += al(2u * n);
     s.plist = wide ? reinterpret_cast<uint16_t *>(p) : nullptr;
+    s.hist = nullptr;
     return s;
   }
 };
@@ -86,7 +88,7 @@ struct CtaScratch {
 // problems; items are visited in strided order by the CTAs.  Inside a realization the source
 // warps claim sources one at a time.
 // ---------------------------------------------------------------------------------------
-template <int BLOCK>
+template <int BLOCK, bool LONG>
 __global__ void __launch_bounds__(BLOCK, 1)
 mc_counts_kernel(const McDev *__restrict__ probs, int nprob, const uint64_t *item_prefix,
                  uint64_t total_items, uint32_t nsw_launch, unsigned char *scratch,
@@ -108,9 +110,10 @@ mc_counts_kernel(const McDev *__restrict__ probs, int nprob, const uint64_t *ite
     const uint32_t n = P.n;
     StepLayout L;
     L.make(n, (uint32_t)(2 * P.m), nsw);
-    uint32_t *rp = reinterpret_cast<uint32_t *>(smem + L.off_rp);
+    uint16_t *rp16 = reinterpret_cast<uint16_t *>(smem + L.off_rp);
+    uint32_t *rp = reinterpret_cast<uint32_t *>(smem + L.off_slots);   // until the sources run
     uint32_t *arc = reinterpret_cast<uint32_t *>(smem + L.off_arc);
-    uint16_t *mw = reinterpret_cast<uint16_t *>(smem + L.off_mw);
+    uint32_t *mwt = reinterpret_cast<uint32_t *>(smem + L.off_mw);
     CtaScratch cs;
     cs.carve(my_scratch, n);
     uint32_t *comp = cs.comp, *cinfo = cs.cinfo, *sel = cs.sel;
@@ -127,7 +130,11 @@ mc_counts_kernel(const McDev *__restrict__ probs, int nprob, const uint64_t *ite
     Realized H{n, rp, arc};
     components(P, H, comp, cinfo);
     if (P.per_row) keep_anchor_component(n, anchor, comp, cinfo);
-    min_lengths(H, mw);
+    if (LONG && !long_lengths(n, ctl->wmax)) {
+      // lengths beyond the problem's declared largest one (the launch chose the form by it)
+      if (threadIdx.x == 0) ctl->err |= kErrInput;
+    }
+    step_tables(H, arc, mwt, LONG);
 
     // sources: every node of a valid component (ascending), alive edges per root for TEPS
     uint32_t *cedges = sel;
@@ -164,7 +171,9 @@ mc_counts_kernel(const McDev *__restrict__ probs, int nprob, const uint64_t *ite
       if (local) atomicAdd(&ctl->edges, local);
       if (lv) atomicAdd(&ctl->verts, lv);
     }
+    for (uint32_t v = threadIdx.x; v <= n; v += blockDim.x) rp16[v] = (uint16_t)rp[v];
     __syncthreads();
+    const StepGraph<uint16_t> SG{n, rp16, arc, mwt};
     const uint32_t nsrc = ctl->nsrc;
 
     // Attempts: compact slots first (wide ones from the start for a length above
@@ -172,6 +181,7 @@ mc_counts_kernel(const McDev *__restrict__ probs, int nprob, const uint64_t *ite
     // (fewer sources at a time), and in FP32 mode a top-two gap under the margin redoes it with
     // FP64 dependencies.  Each can happen once: at most three attempts.
     bool use32 = (P.precision == 1), wide = ctl->wmax > kCompactMaxLen;
+    const uint32_t dbits = dist_bits(n, ctl->wmax) + (LONG ? 1u : 0u);
     const StepSlot s0 = L.slot(smem, 0, n, false);
     for (int attempt = 0; attempt < 3; ++attempt) {
       if (attempt > 0) {
@@ -193,15 +203,15 @@ mc_counts_kernel(const McDev *__restrict__ probs, int nprob, const uint64_t *ite
           if (k >= nsrc) break;
           const uint32_t s = src[k];
           const BcAcc acc{cs.a0, cs.a1, cs.a2};
-          bool ok;
+          StepResult res;
           if (wide)
-            ok = use32 ? source_steps<float, false, true>(H, mw, sl, s, true, acc, err, ovf)
-                       : source_steps<double, false, true>(H, mw, sl, s, true, acc, err, ovf);
+            res = use32 ? source_steps<float, false, true, LONG>(SG, sl, s, dbits, true, acc, err, ovf)
+                        : source_steps<double, false, true, LONG>(SG, sl, s, dbits, true, acc, err, ovf);
           else
-            ok = use32 ? source_steps<float, true, true>(H, mw, sl, s, true, acc, err, ovf)
-                       : source_steps<double, true, true>(H, mw, sl, s, true, acc, err, ovf);
-          if (!ok) break;
-          if (__any_sync(kFull, ovf & kOvfWide)) {
+            res = use32 ? source_steps<float, true, true, LONG>(SG, sl, s, dbits, true, acc, err, ovf)
+                        : source_steps<double, true, true, LONG>(SG, sl, s, dbits, true, acc, err, ovf);
+          if (res == StepResult::failed) break;
+          if (res == StepResult::too_wide) {
             if (lane == 0) atomicOr(&ctl->wide_redo, 1u);
             break;
           }
@@ -292,29 +302,35 @@ __global__ void debug_components_kernel(McDev P, int32_t *comp_out, int32_t *csi
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK, 1)
 debug_sssp_kernel(McDev P, uint32_t r, const int32_t *sources, int32_t nsrc, uint32_t nsw_layout,
-                  uint32_t *dist_out, uint64_t *sigma_out) {
+                  int long_form, uint32_t *dist_out, uint64_t *sigma_out) {
   extern __shared__ __align__(16) unsigned char smem[];
   CtaHead *ctl = reinterpret_cast<CtaHead *>(smem);
   const uint32_t n = P.n, warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
   StepLayout L;
   L.make(n, (uint32_t)(2 * P.m), nsw_layout);
   const uint32_t nsw = L.wide_slots(nsw_layout);
-  uint32_t *rp = reinterpret_cast<uint32_t *>(smem + L.off_rp);
+  uint16_t *rp16 = reinterpret_cast<uint16_t *>(smem + L.off_rp);
+  uint32_t *rp = reinterpret_cast<uint32_t *>(smem + L.off_slots);   // until the sources run
   uint32_t *arc = reinterpret_cast<uint32_t *>(smem + L.off_arc);
-  uint16_t *mw = reinterpret_cast<uint16_t *>(smem + L.off_mw);
+  uint32_t *mwt = reinterpret_cast<uint32_t *>(smem + L.off_mw);
   if (threadIdx.x == 0) { ctl->err = 0; ctl->ovf = 0; ctl->wmax = 1; }
   __syncthreads();
   realize_csr(P, r, rp, arc, ctl);
-  Realized H{n, rp, arc};
-  min_lengths(H, mw);
+  step_tables(Realized{n, rp, arc}, arc, mwt, long_form != 0);
+  for (uint32_t v = threadIdx.x; v <= n; v += blockDim.x) rp16[v] = (uint16_t)rp[v];
   __syncthreads();
+  const StepGraph<uint16_t> SG{n, rp16, arc, mwt};
   const uint32_t k = blockIdx.x * nsw + warp;
   if (warp < nsw && k < (uint32_t)nsrc) {
     const int32_t sv = sources[k];
     const uint32_t s = (sv >= 0 && (uint32_t)sv < n) ? (uint32_t)sv : 0u;
     const StepSlot sl = L.slot(smem, warp, n, true);   // wide slots: 64-bit path counts
     uint32_t err = 0, ovf = 0;
-    source_steps<double, false, true>(H, mw, sl, s, false, BcAcc{}, err, ovf);
+    // 31 distance bits: the dist words keep no levels
+    if (long_form)
+      source_steps<double, false, true, true>(SG, sl, s, 31u, false, BcAcc{}, err, ovf);
+    else
+      source_steps<double, false, true, false>(SG, sl, s, 31u, false, BcAcc{}, err, ovf);
     err = __reduce_or_sync(kFull, err);
     ovf = __reduce_or_sync(kFull, ovf);
     if (lane == 0) {
@@ -324,7 +340,7 @@ debug_sssp_kernel(McDev P, uint32_t r, const int32_t *sources, int32_t nsrc, uin
     for (uint32_t v = lane; v < n; v += 32) {
       const uint32_t d = sl.dist[v] & kMask;
       const bool reached = d < kInf;
-      dist_out[(size_t)k * n + v] = reached ? d : 0xFFFFFFFFu;
+      dist_out[(size_t)k * n + v] = reached ? d >> (long_form ? 1 : 0) : 0xFFFFFFFFu;
       sigma_out[(size_t)k * n + v] = reached ? sl.sig[v] : 0ull;
     }
   }
@@ -356,26 +372,31 @@ size_t mc_cta_scratch_bytes(uint32_t n) { return CtaScratch::bytes(n); }
 
 #define AFC_MC_BLOCKS(X) X(256) X(512) X(1024)
 
-template <int BLOCK>
+template <int BLOCK, bool LONG>
 static cudaError_t launch_counts_t(const McDev *probs_dev, int nprob, const uint64_t *prefix_dev,
                                    uint64_t total_items, uint32_t nsw, uint32_t smem,
                                    uint32_t grid, unsigned char *scratch, size_t stride,
                                    cudaStream_t stream) {
-  cudaFuncSetAttribute(mc_counts_kernel<BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  mc_counts_kernel<BLOCK><<<grid, BLOCK, smem, stream>>>(probs_dev, nprob, prefix_dev,
-                                                         total_items, nsw, scratch, stride);
+  cudaFuncSetAttribute(mc_counts_kernel<BLOCK, LONG>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  mc_counts_kernel<BLOCK, LONG><<<grid, BLOCK, smem, stream>>>(probs_dev, nprob, prefix_dev,
+                                                               total_items, nsw, scratch, stride);
   return cudaGetLastError();
 }
 
-cudaError_t launch_mc_counts(int block, const McDev *probs_dev, int nprob,
+cudaError_t launch_mc_counts(int block, bool long_form, const McDev *probs_dev, int nprob,
                              const uint64_t *prefix_dev, uint64_t total_items,
                              uint32_t source_warps, uint32_t smem_bytes, uint32_t grid,
                              unsigned char *scratch, size_t scratch_stride, cudaStream_t stream) {
   if (source_warps < 1 || source_warps > (uint32_t)block / 32u) return cudaErrorInvalidValue;
-#define AFC_X(B)                                                                       \
-  if (block == B)                                                                      \
-    return launch_counts_t<B>(probs_dev, nprob, prefix_dev, total_items, source_warps, \
-                              smem_bytes, grid, scratch, scratch_stride, stream);
+#define AFC_X(B)                                                                             \
+  if (block == B)                                                                            \
+    return long_form                                                                         \
+               ? launch_counts_t<B, true>(probs_dev, nprob, prefix_dev, total_items,         \
+                                          source_warps, smem_bytes, grid, scratch,           \
+                                          scratch_stride, stream)                            \
+               : launch_counts_t<B, false>(probs_dev, nprob, prefix_dev, total_items,        \
+                                           source_warps, smem_bytes, grid, scratch,          \
+                                           scratch_stride, stream);
   AFC_MC_BLOCKS(AFC_X)
 #undef AFC_X
   return cudaErrorInvalidValue;
@@ -401,24 +422,25 @@ cudaError_t launch_debug_components(const McDev &P, uint32_t r_count, int32_t *c
 
 template <int BLOCK>
 static cudaError_t launch_sssp_t(const McDev &P, uint32_t r, const int32_t *sources, int32_t nsrc,
-                                 uint32_t nsw, uint32_t smem, uint32_t *dist, uint64_t *sigma,
-                                 cudaStream_t stream) {
+                                 uint32_t nsw, bool long_form, uint32_t smem, uint32_t *dist,
+                                 uint64_t *sigma, cudaStream_t stream) {
   StepLayout L;
   L.make((uint32_t)P.n, (uint32_t)(2 * P.m), nsw);
   const int32_t nw = (int32_t)L.wide_slots(nsw);
   const uint32_t grid = (uint32_t)((nsrc + nw - 1) / nw);
   cudaFuncSetAttribute(debug_sssp_kernel<BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  debug_sssp_kernel<BLOCK><<<grid, BLOCK, smem, stream>>>(P, r, sources, nsrc, nsw, dist, sigma);
+  debug_sssp_kernel<BLOCK><<<grid, BLOCK, smem, stream>>>(P, r, sources, nsrc, nsw, long_form ? 1 : 0,
+                                                       dist, sigma);
   return cudaGetLastError();
 }
 
 cudaError_t launch_debug_sssp(int block, const McDev &P, uint32_t r, const int32_t *sources,
-                              int32_t nsrc, uint32_t source_warps, uint32_t smem, uint32_t *dist,
-                              uint64_t *sigma, cudaStream_t stream) {
+                              int32_t nsrc, uint32_t source_warps, bool long_form, uint32_t smem,
+                              uint32_t *dist, uint64_t *sigma, cudaStream_t stream) {
   if (source_warps < 1 || source_warps > (uint32_t)block / 32u) return cudaErrorInvalidValue;
 #define AFC_X(B)                                                                                 \
   if (block == B)                                                                                \
-    return launch_sssp_t<B>(P, r, sources, nsrc, source_warps, smem, dist, sigma, stream);
+    return launch_sssp_t<B>(P, r, sources, nsrc, source_warps, long_form, smem, dist, sigma, stream);
   AFC_MC_BLOCKS(AFC_X)
 #undef AFC_X
   return cudaErrorInvalidValue;

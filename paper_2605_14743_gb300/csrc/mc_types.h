@@ -113,7 +113,8 @@ struct BigGroup {
   double *bc;
   unsigned long long *a1, *a2;
   unsigned long long *best;
-  uint16_t *mw;           // smallest alive incident length per node
+  uint32_t *mwt;          // settle-step kernel: length bounds per node (StepGraph)
+  uint32_t dbits;         // bits of the largest distance key
 };
 
 }  // namespace afc

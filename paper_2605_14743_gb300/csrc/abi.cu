@@ -896,7 +896,7 @@ int afc_absorbing_solve(const afc_chain *chain, const uint32_t *counts, const in
   uint32_t *status = reinterpret_cast<uint32_t *>(ws + L.off_tmp + 256);
   AFC_CUDA(cudaMemsetAsync(status, 0, sizeof(uint32_t), s));
   ChainDev C = chain_dev(chain, counts, c_index, c_list, c);
-  cudaError_t e = launch_solve(C, mu, b, scalars, lu, piv, ws, L, status, s);
+  cudaError_t e = launch_solve(C, mu, b, scalars, lu, piv, ws, L, status, dev_info().smem_optin, s);
   if (e != cudaSuccess) return cuda_fail(e, "solve launch");
   uint32_t st_host = 0;
   AFC_CUDA(cudaMemcpyAsync(&st_host, status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));

@@ -198,12 +198,18 @@ int afc_robust_inner(const afc_chain *chain, const uint32_t *counts, double eps,
   cudaStream_t s = (cudaStream_t)stream;
   uint32_t *status = static_cast<uint32_t *>(workspace);
   AFC_CUDA(cudaMemsetAsync(status, 0, sizeof(uint32_t), s));
+  int32_t *order = nullptr;   // the columns' common order: the caller's workspace has no room
+  if (cudaMallocAsync(&order, sizeof(int32_t) * (size_t)chain->n, s) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return fail(AFC_ENOMEM, "device allocation");
+  }
   cudaError_t e = launch_robust_inner(chain->n, chain->realizations, chain->alpha,
                                       chain->absorb_floor, counts, eps, r_min, support_only ? 1 : 0,
-                                      v, v_bot, 1.0, T, Qstar, status, s);
-  if (e != cudaSuccess) return cuda_fail(e, "robust inner launch");
+                                      v, v_bot, 1.0, order, T, Qstar, status, s);
   uint32_t h = 0;
-  AFC_CUDA(cudaMemcpyAsync(&h, status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&h, status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+  cudaFreeAsync(order, s);
+  if (e != cudaSuccess) return cuda_fail(e, "robust inner launch");
   AFC_CUDA(cudaStreamSynchronize(s));
   if (h) return fail(AFC_EINVAL, "empty uncertainty set: a row's lower bounds exceed 1 - r_min");
   return AFC_OK;
@@ -243,13 +249,16 @@ int afc_robust_value(const afc_chain *chain, const uint32_t *counts, double eps,
   double *mu = reinterpret_cast<double *>(ws + o);
   AFC_CUDA(cudaMemsetAsync(status, 0, sizeof(uint32_t), s));
   AFC_CUDA(cudaMemsetAsync(V, 0, sizeof(double) * (size_t)n, s));
+  const int optin = dev_info().smem_optin;
   // policy iteration: the inner problem's minimiser (or maximiser) at V, then V of that kernel
   int it = 0;
   for (; it < 100; ++it) {
     cudaError_t e = launch_robust_inner(n, chain->realizations, chain->alpha, chain->absorb_floor,
                                         counts, eps, r_min, support_only ? 1 : 0, V, 0.0,
-                                        sense < 0 ? 1.0 : -1.0, T, Qs, status, s);
-    if (e == cudaSuccess) e = launch_robust_eval(n, Qs, A, piv, chain->reward, V, x, diff, status, s);
+                                        sense < 0 ? 1.0 : -1.0, piv, T, Qs, status, s);
+    if (e == cudaSuccess)   // piv: the column order until the LU writes its pivots
+      e = launch_robust_eval(n, Qs, A, piv, chain->reward, chain->s_init, V, x, mu, diff, status,
+                             optin, s);
     if (e != cudaSuccess) return cuda_fail(e, "robust value launch");
     double h_diff = 0.0;
     uint32_t h_st = 0;
@@ -261,7 +270,7 @@ int afc_robust_value(const afc_chain *chain, const uint32_t *counts, double eps,
     if (it > 0 && h_diff <= 1e-13) { ++it; break; }
   }
   if (Qstar) AFC_CUDA(cudaMemcpyAsync(Qstar, Qs, sizeof(double) * nn, cudaMemcpyDeviceToDevice, s));
-  cudaError_t e = launch_robust_star(n, A, piv, chain->s_init, chain->reward, mu, b_star, scalars, s);
+  cudaError_t e = launch_robust_star(n, A, piv, chain->reward, mu, b_star, scalars, s);
   if (e != cudaSuccess) return cuda_fail(e, "robust star launch");
   AFC_CUDA(cudaStreamSynchronize(s));
   if (iterations) *iterations = it;
@@ -345,6 +354,7 @@ int afc_robust_envelope(const afc_chain *chain, const uint32_t *counts, double e
   };
   // Dinkelbach: lambda <- b_v of the kernel optimising s N (e_v - lambda 1) over the set, until
   // it stops moving (that optimum is then 0 and lambda the envelope)
+  const int optin = dev_info().smem_optin;
   for (int outer = 0; outer < 60; ++outer) {
     if (std::find(dk.begin(), dk.end(), 1u) == dk.end()) break;
     AFC_CUDA(cudaMemcpyAsync(d_lambda, lambda.data(), 8 * (size_t)P, cudaMemcpyHostToDevice, s));
@@ -356,7 +366,7 @@ int afc_robust_envelope(const afc_chain *chain, const uint32_t *counts, double e
     for (int it = 0; it < 100; ++it) {
       AFC_CUDA(cudaMemcpyAsync(d_active, pi.data(), 4 * (size_t)P, cudaMemcpyHostToDevice, s));
       e = launch_env_round(n, chain->realizations, chain->alpha, chain->absorb_floor, counts, eps,
-                           r_min, support_only ? 1 : 0, P, B, status, s);
+                           r_min, support_only ? 1 : 0, P, B, chain->s_init, status, optin, s);
       if (e != cudaSuccess) return cuda_fail(e, "envelope round");
       AFC_CUDA(cudaMemcpyAsync(diff.data(), d_diff, 8 * (size_t)P, cudaMemcpyDeviceToHost, s));
       if (int rc = check_status()) return rc;
@@ -368,7 +378,7 @@ int afc_robust_envelope(const afc_chain *chain, const uint32_t *counts, double e
       if (!any) break;
     }
     AFC_CUDA(cudaMemcpyAsync(d_active, dk.data(), 4 * (size_t)P, cudaMemcpyHostToDevice, s));
-    e = launch_env_ratio(n, chain->s_init, P, B, s);
+    e = launch_env_ratio(n, P, B, s);
     if (e != cudaSuccess) return cuda_fail(e, "envelope ratio");
     AFC_CUDA(cudaMemcpyAsync(ratio.data(), d_ratio, 8 * (size_t)P, cudaMemcpyDeviceToHost, s));
     if (int rc = check_status()) return rc;

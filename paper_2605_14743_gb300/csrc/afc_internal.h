@@ -98,7 +98,7 @@ cudaError_t launch_observed_states(int32_t n, const uint32_t *counts, int32_t *c
                                    int32_t *c_list, int32_t *c_dev, cudaStream_t stream);
 cudaError_t launch_solve(const ChainDev &C, double *mu, double *b, double *scalars, double *lu,
                          int32_t *piv, unsigned char *ws, const SolveWs &L, uint32_t *status_dev,
-                         cudaStream_t stream);
+                         int smem_optin, cudaStream_t stream);
 cudaError_t launch_perturb(const ChainDev &C, const afc_perturb_params &pp, const double *mu0,
                            const double *b0, const double *lu0, const int32_t *piv0,
                            uint64_t *counters, uint64_t *pair_flips, uint64_t *shift_hist,
@@ -123,13 +123,13 @@ cudaError_t launch_bootstrap(const ChainDev &C, const int32_t *rec, uint32_t R, 
 cudaError_t launch_robust_inner(int32_t n, uint32_t R, double alpha, double eta,
                                 const uint32_t *counts, double eps, double r_min,
                                 int support_only, const double *v, double v_bot, double vsign,
-                                double *T, double *Qstar, uint32_t *status, cudaStream_t stream);
+                                int32_t *order, double *T, double *Qstar, uint32_t *status,
+                                cudaStream_t stream);
 cudaError_t launch_robust_eval(int32_t n, const double *Qstar, double *A, int32_t *piv,
-                               const double *f, double *V, double *x, double *diff,
-                               uint32_t *status, cudaStream_t stream);
-cudaError_t launch_robust_star(int32_t n, const double *A, const int32_t *piv, const double *s,
-                               const double *f, double *mu, double *b, double *out,
-                               cudaStream_t stream);
+                               const double *f, const double *s, double *V, double *x, double *mu,
+                               double *diff, uint32_t *status, int smem_optin, cudaStream_t stream);
+cudaError_t launch_robust_star(int32_t n, const double *A, const int32_t *piv, const double *f,
+                               double *mu, double *b, double *out, cudaStream_t stream);
 double w1_graph_host(int32_t n, const int32_t *rp, const int32_t *col, const int32_t *eid,
                      const double *x, const double *y);
 
@@ -150,8 +150,8 @@ cudaError_t launch_rank(int32_t n, const double *b, double tie_rel, int32_t k, i
 // p's n-vectors at p * vstride, its n x n matrices at p * n * n
 struct EnvBatch {
   double *Qs, *A;                 // [P][n][n] the inner problem's kernel; I - Q* then its LU
-  double *V, *x, *T, *f;          // [P][vstride]
-  int32_t *piv;                   // [P][vstride]
+  double *V, *x, *T, *f;          // [P][vstride] (T: the inner problem's values, then the visits)
+  int32_t *piv;                   // [P][vstride] the inner problem's column order, then pivots
   size_t vstride;
   const uint32_t *active;         // [P] 1 while the problem iterates
   const double *vsign;            // [P] 1: the adversary minimises, -1: it maximises
@@ -162,10 +162,9 @@ struct EnvBatch {
 cudaError_t launch_env_reward(int32_t n, uint32_t P, const EnvBatch &B, cudaStream_t stream);
 cudaError_t launch_env_round(int32_t n, uint32_t R, double alpha, double eta,
                              const uint32_t *counts, double eps, double r_min, int support_only,
-                             uint32_t P, const EnvBatch &B, uint32_t *status,
-                             cudaStream_t stream);
-cudaError_t launch_env_ratio(int32_t n, const double *s, uint32_t P, const EnvBatch &B,
-                             cudaStream_t stream);
+                             uint32_t P, const EnvBatch &B, const double *s, uint32_t *status,
+                             int smem_optin, cudaStream_t stream);
+cudaError_t launch_env_ratio(int32_t n, uint32_t P, const EnvBatch &B, cudaStream_t stream);
 // robust.cu: maximisers of two discrepancies and the sampled envelopes of a robust search
 cudaError_t launch_robust_summary(int32_t n, int32_t count, const double *rows, const double *b0,
                                   const double *d1, const double *d2, int32_t *arg, double *lo,

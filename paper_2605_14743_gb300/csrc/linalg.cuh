@@ -314,64 +314,10 @@ __device__ inline bool lu_factor_blocked_t(T *A, int32_t c, int32_t lda, int32_t
   return true;
 }
 
-// A x = b with factors of type F (lu_factor_blocked_t), b and x in FP64 (in place).
-template <typename F>
-__device__ inline void lu_solve_t(const F *LU, int32_t c, int32_t lda, const int32_t *piv,
-                                  double *b, LinScratch s) {
-  if (threadIdx.x == 0)
-    for (int32_t k = 0; k < c; ++k) {
-      const int32_t p = piv[k];
-      if (p != k) { const double t = b[k]; b[k] = b[p]; b[p] = t; }
-    }
-  __syncthreads();
-  for (int32_t k = 0; k < c; ++k) {
-    const double yk = b[k];
-    for (int32_t i = k + 1 + threadIdx.x; i < c; i += blockDim.x)
-      b[i] = fma(-(double)LU[(size_t)i * lda + k], yk, b[i]);
-    __syncthreads();
-  }
-  for (int32_t k = c - 1; k >= 0; --k) {
-    if (threadIdx.x == 0) s.bcast[0] = b[k] / (double)LU[(size_t)k * lda + k];
-    __syncthreads();
-    const double xk = s.bcast[0];
-    for (int32_t i = threadIdx.x; i < k; i += blockDim.x)
-      b[i] = fma(-(double)LU[(size_t)i * lda + k], xk, b[i]);
-    if (threadIdx.x == 0) b[k] = xk;
-    __syncthreads();
-  }
-}
-
-// A^T x = b with factors of type F, FP64 vectors (in place).
-template <typename F>
-__device__ inline void lu_solve_transposed_t(const F *LU, int32_t c, int32_t lda,
-                                             const int32_t *piv, double *b, LinScratch s) {
-  for (int32_t k = 0; k < c; ++k) {
-    if (threadIdx.x == 0) s.bcast[0] = b[k] / (double)LU[(size_t)k * lda + k];
-    __syncthreads();
-    const double zk = s.bcast[0];
-    for (int32_t i = k + 1 + threadIdx.x; i < c; i += blockDim.x)
-      b[i] = fma(-(double)LU[(size_t)k * lda + i], zk, b[i]);
-    if (threadIdx.x == 0) b[k] = zk;
-    __syncthreads();
-  }
-  for (int32_t k = c - 1; k >= 0; --k) {
-    const double wk = b[k];
-    for (int32_t i = threadIdx.x; i < k; i += blockDim.x)
-      b[i] = fma(-(double)LU[(size_t)k * lda + i], wk, b[i]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0)
-    for (int32_t k = c - 1; k >= 0; --k) {
-      const int32_t p = piv[k];
-      if (p != k) { const double t = b[k]; b[k] = b[p]; b[p] = t; }
-    }
-  __syncthreads();
-}
-
 // Blocked triangular solves with factors of type F on FP64 vectors (in place), for factors in
 // device memory: per 32-row block, warp 0 solves the diagonal block with shuffles, then the
 // CTA updates the remaining rows with the block's solution.  Two barriers per block instead
-// of one per row.  Same results as lu_solve_t / lu_solve_transposed_t up to rounding order.
+// of one per row.
 template <typename F>
 __device__ inline void lu_solve_blocked_t(const F *LU, int32_t c, int32_t lda, const int32_t *piv,
                                           double *b) {

@@ -6,11 +6,13 @@
 //                        support, or on every j) with sum_j q_ij <= 1 - r_min.  A warp per row
 //                        solves the LP exactly: every entry starts at its lower bound, then the
 //                        budget goes to the entries in ascending order of v_j - v_bot (ties by
-//                        j) while that coefficient is negative, each up to its upper bound.
-//   eval_kernel          one CTA: A = I - Q*, V = A^-1 f (blocked FP64 LU with partial pivoting) and
-//                        the change of V; the robust value comes from policy iteration on the
-//                        host (inner problem at V, evaluate, until V stops changing)
-//   star_kernel          the AFC of the scenario kernel: A^T mu = s with the last factors
+//                        j) while that coefficient is negative, each up to its upper bound.  The
+//                        order is the same for every row (robust_order_kernel).
+//   launch_robust_eval   A = I - Q*, its LU over the whole GPU (dense_lu.cu) with f and s in the
+//                        elimination, V = A^-1 f and the change of V; the robust value comes from
+//                        policy iteration on the host (inner problem at V, evaluate, until V stops
+//                        changing)
+//   star_kernel          the AFC of the scenario kernel: mu A = s from the last elimination
 // Host (Sec. 9 robust experiment): the Wasserstein-1 distance between two node distributions
 // under the base graph's hop metric.
 //
@@ -26,6 +28,7 @@
 #include <cuda_runtime.h>
 
 #include "afc_internal.h"
+#include "dense_lu.cuh"
 #include "linalg.cuh"
 
 namespace afc {
@@ -53,103 +56,147 @@ __device__ __forceinline__ double warp_sum_d(double x) {
   return x;
 }
 
+// v ordered like its value as an unsigned integer (NaN last)
+__device__ __forceinline__ unsigned long long sortable(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  return v != v ? ~0ull : (b >> 63) ? ~b : b | 0x8000000000000000ull;
+}
+
+// order[] = the columns with a negative coefficient cf_j = vsign v_j - vb in ascending (cf, j) and
+// *nneg how many: every row of the inner problem spends its budget in this order, so it is made
+// once per call (a warp per column counts the columns before it, in integer compares).
+__device__ void order_columns(int32_t n, const double *v, double vb, double vsign, int32_t *order,
+                              uint32_t warp, uint32_t nwarps) {
+  const uint32_t lane = threadIdx.x & 31u;
+  for (uint32_t j = warp; j < (uint32_t)n; j += nwarps) {
+    const double cj = vsign * v[j] - vb;
+    if (!(cj < 0.0)) continue;
+    const unsigned long long kj = sortable(cj);
+    uint32_t before = 0;
+    for (uint32_t i = lane; i < (uint32_t)n; i += 32) {
+      const unsigned long long ki = sortable(vsign * v[i] - vb);
+      before += (ki < kj || (ki == kj && i < j)) ? 1u : 0u;
+    }
+    before = __reduce_add_sync(0xFFFFFFFFu, before);
+    if (lane == 0) order[before] = (int32_t)j;
+  }
+}
+
+// How many columns order_columns placed: the columns with a negative coefficient.
+__device__ __forceinline__ uint32_t count_negative(int32_t n, const double *v, double vb, double vsign) {
+  uint32_t k = 0;
+  for (int32_t j = threadIdx.x & 31; j < n; j += 32) k += vsign * v[j] - vb < 0.0 ? 1u : 0u;
+  return __reduce_add_sync(0xFFFFFFFFu, k);
+}
+
 // Row-wise inner problem (warp per row, rows warp, warp + nwarps, ...) at the continuation
-// value vsign * (v, v_bot).
+// value vsign * (v, v_bot): the budget is handed out 32 columns of the common order at a time, by
+// a prefix sum of their caps.  (Searching the next column for each row cost n per column: 550 us
+// at n = 500.)
 __device__ void inner_rows(int32_t n, uint32_t R, double alpha, double eta,
                            const uint32_t *counts, double eps, double r_min, int support_only,
-                           const double *v, double v_bot, double vsign, double *T, double *Qstar,
-                           uint32_t *status, uint32_t warp, uint32_t nwarps) {
+                           const double *v, double v_bot, double vsign, const int32_t *order,
+                           double *T, double *Qstar, uint32_t *status, uint32_t warp,
+                           uint32_t nwarps) {
   const uint32_t lane = threadIdx.x & 31u;
   const size_t stride = (size_t)n + 1;
   const double vb = vsign * v_bot;
+  uint32_t nneg = 0xFFFFFFFFu;
   for (uint32_t i = warp; i < (uint32_t)n; i += nwarps) {
+    if (nneg == 0xFFFFFFFFu) nneg = count_negative(n, v, vb, vsign);
     const uint32_t *row = counts + (size_t)i * stride;
     const double scale = row_scale_warp(row, n, R, alpha, eta);
     double *qs = Qstar ? Qstar + (size_t)i * n : nullptr;
     // every entry at its lower bound
     double base = 0.0, low = 0.0;
     for (int32_t j = lane; j < n; j += 32) {
-      const double q = scale * (double)row[j];
-      const double l = q > eps ? q - eps : 0.0;
-      base += l * (vsign * v[j] - vb);
-      low += l;
+      const uint32_t k = row[j];
+      double l = 0.0;
+      if (k) {
+        const double q = scale * (double)k;
+        l = q > eps ? q - eps : 0.0;
+        base += l * (vsign * v[j] - vb);
+        low += l;
+      }
       if (qs) qs[j] = l;
     }
     base = warp_sum_d(base);
     low = warp_sum_d(low);
-    __syncwarp();   // the lower bounds written by every lane, before lane 0 adds to them
+    __syncwarp();   // the lower bounds written by every lane, before the budget is added
     double budget = (1.0 - r_min) - low;
     if (budget < -1e-12) {
       if (lane == 0) atomicOr(status, kErrInput);   // U_i is empty
       budget = 0.0;
     }
     // the budget to the most negative coefficients first, each entry up to its upper bound
-    double acc = 0.0, last_c = -INFINITY;
-    int32_t last_j = -1;
-    while (budget > 0.0) {
-      double bc = 0.0;
-      int32_t bj = 0x7FFFFFFF;
-      double bcap = 0.0;
-      for (int32_t j = lane; j < n; j += 32) {
-        const double cf = vsign * v[j] - vb;
-        if (!(cf < 0.0)) continue;
-        if (cf < last_c || (cf == last_c && j <= last_j)) continue;   // already filled
+    double acc = 0.0;
+    for (uint32_t k0 = 0; k0 < nneg && budget > 0.0; k0 += 32) {
+      const uint32_t k = k0 + lane;
+      int32_t j = 0;
+      double cap = 0.0;
+      if (k < nneg) {
+        j = order[k];
         const double q = scale * (double)row[j];
-        double cap;
         if (q > 0.0) cap = fmin(q + eps, 1.0) - (q > eps ? q - eps : 0.0);
-        else cap = support_only ? 0.0 : fmin(eps, 1.0);
-        if (!(cap > 0.0)) continue;
-        if (bj == 0x7FFFFFFF || cf < bc || (cf == bc && j < bj)) { bc = cf; bj = j; bcap = cap; }
+        else if (!support_only) cap = fmin(eps, 1.0);
+        if (!(cap > 0.0)) cap = 0.0;
       }
+      if (!__any_sync(0xFFFFFFFFu, cap > 0.0)) continue;
+      double incl = cap;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const double oc = __shfl_xor_sync(0xFFFFFFFFu, bc, o);
-        const int32_t oj = __shfl_xor_sync(0xFFFFFFFFu, bj, o);
-        const double ocap = __shfl_xor_sync(0xFFFFFFFFu, bcap, o);
-        if (oj != 0x7FFFFFFF && (bj == 0x7FFFFFFF || oc < bc || (oc == bc && oj < bj))) {
-          bc = oc; bj = oj; bcap = ocap;
-        }
+      for (int o = 1; o < 32; o <<= 1) {
+        const double y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= (uint32_t)o) incl += y;
       }
-      if (bj == 0x7FFFFFFF) break;
-      const double d = fmin(bcap, budget);
-      acc += d * bc;
-      budget -= d;
-      if (qs && lane == 0) qs[bj] += d;
-      last_c = bc;
-      last_j = bj;
+      double before = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
+      if (lane == 0) before = 0.0;
+      const double d = fmin(cap, fmax(budget - before, 0.0));
+      if (d > 0.0) {
+        acc += d * (vsign * v[j] - vb);
+        if (qs) qs[j] += d;
+      }
+      budget -= __shfl_sync(0xFFFFFFFFu, incl, 31);
     }
+    acc = warp_sum_d(acc);
     if (lane == 0) T[i] = vsign * (vb + base + acc);
   }
+}
+
+__global__ void robust_order_kernel(int32_t n, const double *v, double v_bot, double vsign,
+                                    int32_t *order) {
+  order_columns(n, v, vsign * v_bot, vsign, order, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                (gridDim.x * blockDim.x) >> 5);
 }
 
 __global__ void robust_inner_kernel(int32_t n, uint32_t R, double alpha, double eta,
                                     const uint32_t *counts, double eps, double r_min,
                                     int support_only, const double *v, double v_bot, double vsign,
-                                    double *T, double *Qstar, uint32_t *status) {
-  inner_rows(n, R, alpha, eta, counts, eps, r_min, support_only, v, v_bot, vsign, T, Qstar,
+                                    const int32_t *order, double *T, double *Qstar,
+                                    uint32_t *status) {
+  inner_rows(n, R, alpha, eta, counts, eps, r_min, support_only, v, v_bot, vsign, order, T, Qstar,
              status, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
              (gridDim.x * blockDim.x) >> 5);
 }
 
-__global__ void build_a_kernel(int32_t n, const double *Qstar, double *A) {
+// A = I - Q*, and the right-hand sides the elimination carries: x = f (1 when null), mu = s
+// (uniform when null).
+__global__ void build_a_kernel(int32_t n, const double *Qstar, const double *f, const double *s,
+                               double *A, double *x, double *mu) {
   const size_t nn = (size_t)n * n;
-  for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < nn;
-       k += (size_t)gridDim.x * blockDim.x)
+  const size_t k0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  for (size_t k = k0; k < nn; k += (size_t)gridDim.x * blockDim.x)
     A[k] = ((k / n) == (k % n) ? 1.0 : 0.0) - Qstar[k];
+  for (size_t k = k0; k < (size_t)n; k += (size_t)gridDim.x * blockDim.x) {
+    x[k] = f ? f[k] : 1.0;
+    mu[k] = s ? s[k] : 1.0 / (double)n;
+  }
 }
 
-// One CTA of 256 threads: factor A (the blocked LU: the matrix is in device memory), V_new =
-// A^-1 f (f = 1 when null), diff = max |V_new - V|, V <- V_new.
-__device__ void eval_body(int32_t n, double *A, int32_t *piv, const double *f, double *V,
-                          double *x, double *diff, uint32_t *status, LinScratch ls, double *red,
-                          double *tiles) {
-  if (!lu_factor_blocked(A, n, n, piv, ls, tiles)) {
-    if (threadIdx.x == 0) { atomicOr(status, kErrSolve); *diff = 0.0; }
-    return;
-  }
-  for (int32_t i = threadIdx.x; i < n; i += blockDim.x) x[i] = f ? f[i] : 1.0;
-  __syncthreads();
-  lu_solve(A, n, n, piv, x, ls);
+// One CTA: V_new = U^-1 x (x = L^-1 P f from the elimination), diff = max |V_new - V| relative to
+// max |V_new|, V <- V_new.
+__device__ void eval_body(int32_t n, const double *A, double *V, double *x, double *diff,
+                          TriScratch &tri, double *red) {
+  upper_solve(A, n, x, tri);
   double m = 0.0, scale = 1.0;
   for (int32_t i = threadIdx.x; i < n; i += blockDim.x) {
     m = fmax(m, fabs(x[i] - V[i]));
@@ -161,33 +208,21 @@ __device__ void eval_body(int32_t n, double *A, int32_t *piv, const double *f, d
   if (threadIdx.x == 0) *diff = m / scale;
 }
 
-__global__ void __launch_bounds__(256, 1)
-eval_kernel(int32_t n, double *A, int32_t *piv, const double *f, double *V, double *x,
-            double *diff, uint32_t *status) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ double sval[33];
-  __shared__ int32_t sidx[32];
-  __shared__ double sb[2];
-  __shared__ int32_t sflag[1];
+__global__ void __launch_bounds__(1024, 1)
+eval_kernel(int32_t n, const double *A, double *V, double *x, double *diff) {
+  __shared__ TriScratch tri;
   __shared__ double red[33];
-  LinScratch ls{sval, sidx, sb, sflag};
-  eval_body(n, A, piv, f, V, x, diff, status, ls, red, reinterpret_cast<double *>(smem));
+  eval_body(n, A, V, x, diff, tri, red);
 }
 
-// The AFC of the scenario kernel from the factors of the last evaluation: A^T mu = s,
-// out[0] = E_s[T] = sum mu, out[1] = b . f (f = 1 when null gives 1).
+// The AFC of the scenario kernel from the last elimination (mu = s U^-1): L^T mu, out[0] = E_s[T]
+// = sum mu, out[1] = b . f (f = 1 when null gives 1).
 __global__ void __launch_bounds__(1024, 1)
-star_kernel(int32_t n, const double *A, const int32_t *piv, const double *s, const double *f,
-            double *mu, double *b, double *out) {
-  __shared__ double sval[33];
-  __shared__ int32_t sidx[32];
-  __shared__ double sb[2];
-  __shared__ int32_t sflag[1];
+star_kernel(int32_t n, const double *A, const int32_t *piv, const double *f, double *mu, double *b,
+            double *out) {
+  __shared__ TriScratch tri;
   __shared__ double red[33];
-  LinScratch ls{sval, sidx, sb, sflag};
-  for (int32_t i = threadIdx.x; i < n; i += blockDim.x) mu[i] = s ? s[i] : 1.0 / (double)n;
-  __syncthreads();
-  lu_solve_transposed(A, n, n, piv, mu, ls);
+  lower_t_solve(A, n, piv, mu, tri);
   double t = 0.0, tf = 0.0;
   for (int32_t i = threadIdx.x; i < n; i += blockDim.x) {
     t += mu[i];
@@ -201,6 +236,13 @@ star_kernel(int32_t n, const double *A, const int32_t *piv, const double *s, con
 
 // ---- batched robust problems (the envelopes): problem p's arrays at p times the stride ----
 
+__global__ void order_batched_kernel(int32_t n, const EnvBatch B) {
+  const uint32_t p = blockIdx.y;
+  if (!B.active[p]) return;
+  order_columns(n, B.V + p * B.vstride, 0.0, B.vsign[p], B.piv + p * B.vstride,
+                (blockIdx.x * blockDim.x + threadIdx.x) >> 5, (gridDim.x * blockDim.x) >> 5);
+}
+
 // inner problem of every active problem (blockIdx.y = problem)
 __global__ void inner_batched_kernel(int32_t n, uint32_t R, double alpha, double eta,
                                      const uint32_t *counts, double eps, double r_min,
@@ -209,48 +251,47 @@ __global__ void inner_batched_kernel(int32_t n, uint32_t R, double alpha, double
   if (!B.active[p]) return;
   const size_t nn = (size_t)n * n;
   inner_rows(n, R, alpha, eta, counts, eps, r_min, support_only, B.V + p * B.vstride, 0.0,
-             B.vsign[p], B.T + p * B.vstride, B.Qs + p * nn, status,
+             B.vsign[p], B.piv + p * B.vstride, B.T + p * B.vstride, B.Qs + p * nn, status,
              (blockIdx.x * blockDim.x + threadIdx.x) >> 5, (gridDim.x * blockDim.x) >> 5);
 }
 
-// one CTA per active problem: A = I - Q*, its LU, V <- A^-1 f, diff
-__global__ void __launch_bounds__(256, 1)
-eval_batched_kernel(int32_t n, const EnvBatch B, uint32_t *status) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ double sval[33];
-  __shared__ int32_t sidx[32];
-  __shared__ double sb[2];
-  __shared__ int32_t sflag[1];
-  __shared__ double red[33];
-  const uint32_t p = blockIdx.x;
+// every active problem's A = I - Q* and right-hand sides: x = f_p, and T (the inner values are no
+// longer needed) = s
+__global__ void build_a_batched_kernel(int32_t n, const EnvBatch B, const double *s) {
+  const uint32_t p = blockIdx.y;
   if (!B.active[p]) return;
-  LinScratch ls{sval, sidx, sb, sflag};
   const size_t nn = (size_t)n * n;
   const double *Qs = B.Qs + p * nn;
   double *A = B.A + p * nn;
-  for (size_t k = threadIdx.x; k < nn; k += blockDim.x)
+  const size_t k0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  for (size_t k = k0; k < nn; k += (size_t)gridDim.x * blockDim.x)
     A[k] = ((k / n) == (k % n) ? 1.0 : 0.0) - Qs[k];
-  __syncthreads();
-  eval_body(n, A, B.piv + p * B.vstride, B.f + p * B.vstride, B.V + p * B.vstride,
-            B.x + p * B.vstride, B.diff + p, status, ls, red, reinterpret_cast<double *>(smem));
+  for (size_t k = k0; k < (size_t)n; k += (size_t)gridDim.x * blockDim.x) {
+    B.x[p * B.vstride + k] = B.f[p * B.vstride + k];
+    B.T[p * B.vstride + k] = s ? s[k] : 1.0 / (double)n;
+  }
 }
 
-// one CTA per active problem: the visits mu of its kernel (A^T mu = s from the last factors),
-// ratio[p] = mu_v / sum mu = b_v for the problem's node v
-__global__ void __launch_bounds__(1024, 1)
-star_batched_kernel(int32_t n, const double *s, const EnvBatch B) {
-  __shared__ double sval[33];
-  __shared__ int32_t sidx[32];
-  __shared__ double sb[2];
-  __shared__ int32_t sflag[1];
+// one CTA per active problem: V <- U^-1 x, diff
+__global__ void __launch_bounds__(1024, 1) eval_batched_kernel(int32_t n, const EnvBatch B) {
+  __shared__ TriScratch tri;
   __shared__ double red[33];
   const uint32_t p = blockIdx.x;
   if (!B.active[p]) return;
-  LinScratch ls{sval, sidx, sb, sflag};
-  double *mu = B.x + p * B.vstride;
-  for (int32_t i = threadIdx.x; i < n; i += blockDim.x) mu[i] = s ? s[i] : 1.0 / (double)n;
-  __syncthreads();
-  lu_solve_transposed(B.A + p * (size_t)n * n, n, n, B.piv + p * B.vstride, mu, ls);
+  eval_body(n, B.A + p * (size_t)n * n, B.V + p * B.vstride, B.x + p * B.vstride, B.diff + p, tri,
+            red);
+}
+
+// one CTA per active problem: the visits mu of its kernel (L^T mu from the last elimination),
+// ratio[p] = mu_v / sum mu = b_v for the problem's node v
+__global__ void __launch_bounds__(1024, 1)
+star_batched_kernel(int32_t n, const EnvBatch B) {
+  __shared__ TriScratch tri;
+  __shared__ double red[33];
+  const uint32_t p = blockIdx.x;
+  if (!B.active[p]) return;
+  double *mu = B.T + p * B.vstride;
+  lower_t_solve(B.A + p * (size_t)n * n, n, B.piv + p * B.vstride, mu, tri);
   double t = 0.0;
   for (int32_t i = threadIdx.x; i < n; i += blockDim.x) t += mu[i];
   const double T = block_sum(t, red);
@@ -281,46 +322,54 @@ cudaError_t launch_env_reward(int32_t n, uint32_t P, const EnvBatch &B, cudaStre
 
 cudaError_t launch_env_round(int32_t n, uint32_t R, double alpha, double eta,
                              const uint32_t *counts, double eps, double r_min, int support_only,
-                             uint32_t P, const EnvBatch &B, uint32_t *status,
-                             cudaStream_t stream) {
+                             uint32_t P, const EnvBatch &B, const double *s, uint32_t *status,
+                             int smem_optin, cudaStream_t stream) {
   const dim3 grid((unsigned)std::min<int64_t>(((int64_t)n + 7) / 8, 1024), P);
+  order_batched_kernel<<<grid, 256, 0, stream>>>(n, B);
   inner_batched_kernel<<<grid, 256, 0, stream>>>(n, R, alpha, eta, counts, eps, r_min,
                                                  support_only, B, status);
-  eval_batched_kernel<<<P, 256, sizeof(double) * lu_blocked_smem_doubles(), stream>>>(n, B,
-                                                                                     status);
+  const dim3 agrid((unsigned)std::min<int64_t>(((int64_t)n * n + 1023) / 1024, 1024), P);
+  build_a_batched_kernel<<<agrid, 256, 0, stream>>>(n, B, s);
+  const LuBatch L{B.A, (size_t)n * n, B.piv, B.vstride, B.T, B.x, B.active, status};
+  cudaError_t e = launch_lu(L, n, (int32_t)P, smem_optin, stream);
+  if (e != cudaSuccess) return e;
+  eval_batched_kernel<<<P, 1024, 0, stream>>>(n, B);
   return cudaGetLastError();
 }
 
-cudaError_t launch_env_ratio(int32_t n, const double *s, uint32_t P, const EnvBatch &B,
-                             cudaStream_t stream) {
-  star_batched_kernel<<<P, 1024, 0, stream>>>(n, s, B);
+cudaError_t launch_env_ratio(int32_t n, uint32_t P, const EnvBatch &B, cudaStream_t stream) {
+  star_batched_kernel<<<P, 1024, 0, stream>>>(n, B);
   return cudaGetLastError();
 }
 
 cudaError_t launch_robust_inner(int32_t n, uint32_t R, double alpha, double eta,
                                 const uint32_t *counts, double eps, double r_min,
                                 int support_only, const double *v, double v_bot, double vsign,
-                                double *T, double *Qstar, uint32_t *status, cudaStream_t stream) {
+                                int32_t *order, double *T, double *Qstar, uint32_t *status,
+                                cudaStream_t stream) {
   const int grid = (int)std::min<int64_t>(((int64_t)n + 7) / 8, 1024);
+  robust_order_kernel<<<grid, 256, 0, stream>>>(n, v, v_bot, vsign, order);
   robust_inner_kernel<<<grid, 256, 0, stream>>>(n, R, alpha, eta, counts, eps, r_min,
-                                                support_only, v, v_bot, vsign, T, Qstar, status);
+                                                support_only, v, v_bot, vsign, order, T, Qstar,
+                                                status);
   return cudaGetLastError();
 }
 
 cudaError_t launch_robust_eval(int32_t n, const double *Qstar, double *A, int32_t *piv,
-                               const double *f, double *V, double *x, double *diff,
-                               uint32_t *status, cudaStream_t stream) {
+                               const double *f, const double *s, double *V, double *x, double *mu,
+                               double *diff, uint32_t *status, int smem_optin, cudaStream_t stream) {
   const int grid = (int)std::min<int64_t>(((int64_t)n * n + 255) / 256, 4096);
-  build_a_kernel<<<grid, 256, 0, stream>>>(n, Qstar, A);
-  eval_kernel<<<1, 256, sizeof(double) * lu_blocked_smem_doubles(), stream>>>(n, A, piv, f, V, x,
-                                                                              diff, status);
+  build_a_kernel<<<grid, 256, 0, stream>>>(n, Qstar, f, s, A, x, mu);
+  const LuBatch B{A, 0, piv, 0, mu, x, nullptr, status};
+  cudaError_t e = launch_lu(B, n, 1, smem_optin, stream);
+  if (e != cudaSuccess) return e;
+  eval_kernel<<<1, 1024, 0, stream>>>(n, A, V, x, diff);
   return cudaGetLastError();
 }
 
-cudaError_t launch_robust_star(int32_t n, const double *A, const int32_t *piv, const double *s,
-                               const double *f, double *mu, double *b, double *out,
-                               cudaStream_t stream) {
-  star_kernel<<<1, 1024, 0, stream>>>(n, A, piv, s, f, mu, b, out);
+cudaError_t launch_robust_star(int32_t n, const double *A, const int32_t *piv, const double *f,
+                               double *mu, double *b, double *out, cudaStream_t stream) {
+  star_kernel<<<1, 1024, 0, stream>>>(n, A, piv, f, mu, b, out);
   return cudaGetLastError();
 }
 

@@ -2,6 +2,7 @@
 // FP64 absorbing-chain solve on the observed centre states C (Sec. 4 eqs. fundamental,
 // visits, expected-length, afc-def; Sec. 6.4 eq. mr-inner-product; Sec. 8.2 floor), plus the
 // visit-gap certificates of Sec. 5.5 (eqs. pm-gap, sharp-gap).
+// The elimination runs over the whole GPU with both right-hand sides in it (dense_lu.cu).
 //
 // With the columns of U = V \ C zero, N = (I - Q)^-1 has the block form [[I, Q_UC N_CC],
 // [0, N_CC]] in (U, C) order, so mu_U = s_U and mu_C (I - Q_CC) = s_C + s_U Q_UC.
@@ -10,6 +11,7 @@
 #include <cuda_runtime.h>
 
 #include "afc_internal.h"
+#include "dense_lu.cuh"
 #include "linalg.cuh"
 
 namespace afc {
@@ -20,7 +22,16 @@ __global__ void column_flags_kernel(int32_t n, const uint32_t *counts, uint32_t 
   if (j >= n) return;
   const size_t stride = (size_t)n + 1;
   uint32_t any = 0;
-  for (int32_t i = blockIdx.y; i < n; i += gridDim.y) any |= counts[(size_t)i * stride + j];
+  int32_t i = blockIdx.y;
+  // eight independent loads in flight (one pass over the count matrix, bound by its latency)
+  for (; i + 7 * (int32_t)gridDim.y < n; i += 8 * (int32_t)gridDim.y) {
+    uint32_t v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = counts[(size_t)(i + u * (int32_t)gridDim.y) * stride + j];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) any |= v[u];
+  }
+  for (; i < n; i += gridDim.y) any |= counts[(size_t)i * stride + j];
   if (any) flags[j] = 1u;
 }
 
@@ -160,10 +171,10 @@ __global__ void exclusive_scan_kernel(int32_t n, const int32_t *in, int32_t *out
   if (threadIdx.x == 0) out[n] = base;
 }
 
-// Writes the sparse rows (C positions ascending, then the absorbing column as position c)
-// and scatters A = I - Q_CC and y = s_C + s_U Q_UC.
+// Writes the sparse rows (C positions ascending, then the absorbing column as position c) and the
+// dense rows of A = I - Q_CC.  A warp per row, four windows of 32 columns loaded at a time.
 __global__ void row_fill_kernel(ChainDev C, const double *rowscale, const int32_t *nzptr,
-                                int32_t *nzcol, double *nzval, double *A, double *y) {
+                                int32_t *nzcol, double *nzval, double *A, double *t) {
   const int32_t n = C.n, c = C.c;
   const size_t stride = (size_t)n + 1;
   const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31u;
@@ -171,104 +182,145 @@ __global__ void row_fill_kernel(ChainDev C, const double *rowscale, const int32_
   for (int32_t i = warp; i < n; i += nwarps) {
     const uint32_t *row = C.counts + (size_t)i * stride;
     const double scale = rowscale[2 * i], r = rowscale[2 * i + 1];
-    const double si = C.s ? C.s[i] : 1.0 / (double)n;
     const int32_t pi = C.c_index[i];
+    double *ar = pi >= 0 ? A + (size_t)pi * c : nullptr;
+    if (ar) {
+      for (int32_t j = (int32_t)lane; j < c; j += 32) ar[j] = j == pi ? 1.0 : 0.0;
+      if (lane == 0) t[pi] = 1.0;   // the right-hand side of N 1
+      __syncwarp();
+    }
     int32_t out = nzptr[i];
-    for (int32_t j0 = 0; j0 < n; j0 += 32) {
-      const int32_t j = j0 + lane;
-      const uint32_t v = j < n ? row[j] : 0u;
-      const uint32_t ball = __ballot_sync(0xFFFFFFFFu, v != 0);
-      if (v) {
-        const int32_t pos = out + __popc(ball & ((1u << lane) - 1u));
-        const int32_t pj = C.c_index[j];
-        const double q = scale * (double)v;
-        nzcol[pos] = pj;
-        nzval[pos] = q;
-        if (pi >= 0) A[(size_t)pi * c + pj] -= q;  // distinct (pi, pj) per lane: no race
-        else atomicAdd(&y[pj], si * q);
+    for (int32_t j0 = 0; j0 < n; j0 += 128) {
+      uint32_t v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int32_t j = j0 + 32 * u + (int32_t)lane;
+        v[u] = j < n ? row[j] : 0u;
       }
-      out += __popc(ball);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const uint32_t ball = __ballot_sync(0xFFFFFFFFu, v[u] != 0);
+        if (v[u]) {
+          const int32_t pos = out + __popc(ball & ((1u << lane) - 1u));
+          const int32_t pj = C.c_index[j0 + 32 * u + (int32_t)lane];
+          const double q = scale * (double)v[u];
+          nzcol[pos] = pj;
+          nzval[pos] = q;
+          if (ar) ar[pj] -= q;   // one lane per column
+        }
+        out += __popc(ball);
+      }
     }
     if (lane == 0) {
       nzcol[out] = c;  // absorbing column
       nzval[out] = r;
-      if (pi >= 0) atomicAdd(&y[pi], si);
     }
   }
 }
 
-__global__ void identity_kernel(double *A, int32_t c) {
-  const size_t total = (size_t)c * c;
-  for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < total;
-       k += (size_t)gridDim.x * blockDim.x)
-    A[k] = (k / c == k % c) ? 1.0 : 0.0;
-}
-
-// ---- factor + solves + finalise (one CTA) -----------------------------------------------------
-__global__ void __launch_bounds__(1024, 1)
-chain_solve_kernel(ChainDev C, double *A, int32_t *piv, double *y, double *t,
-                   const double *rowscale, const int32_t *nzptr, const int32_t *nzcol,
-                   const double *nzval, double *mu, double *b, double *scalars,
-                   uint32_t *status) {
-  __shared__ double sval[33];
-  __shared__ int32_t sidx[32];
-  __shared__ double sb[2];
-  __shared__ int32_t sflag[1];
-  __shared__ double red[33];
-  LinScratch ls{sval, sidx, sb, sflag};
+// s_U Q_UC: partial sums over the rows [chunk i0, chunk i1) of the grid's y dimension, a thread per
+// observed state, rows ascending (a fixed order; atomics on c addresses took 44 us at n = 1,000).
+__global__ void u_rows_kernel(ChainDev C, const double *rowscale, double *part) {
   const int32_t n = C.n, c = C.c;
-  bool ok = true;
-  if (c > 0) {
-    ok = lu_factor(A, c, c, piv, ls);
-    if (ok) {
-      lu_solve_transposed(A, c, c, piv, y, ls);                  // mu_C
-      for (int32_t k = threadIdx.x; k < c; k += blockDim.x) t[k] = 1.0;
-      __syncthreads();
-      lu_solve(A, c, c, piv, t, ls);                             // (N 1) on C
-    }
+  const int32_t pj = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x);
+  if (pj >= c) return;
+  const size_t stride = (size_t)n + 1;
+  const int32_t per = (n + (int32_t)gridDim.y - 1) / (int32_t)gridDim.y;
+  const int32_t i0 = (int32_t)blockIdx.y * per, i1 = min(n, i0 + per);
+  const uint32_t *colp = C.counts + C.c_list[pj];
+  const double unif = 1.0 / (double)n;
+  double acc = 0.0;
+  for (int32_t i = i0; i < i1; i += 8) {
+    uint32_t v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      v[u] = i + u < i1 && C.c_index[i + u] < 0 ? colp[(size_t)(i + u) * stride] : 0u;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (v[u]) acc = fma((C.s ? C.s[i + u] : unif) * rowscale[2 * (i + u)], (double)v[u], acc);
   }
-  if (!ok) {
-    if (threadIdx.x == 0) *status |= kErrSolve;
-    return;
-  }
-  // mu, E[T], b, b_f; max (N 1) including the U rows: 1 + sum_j Q_ij (N 1)_j
-  double part = 0.0, tmax = 0.0;
+  part[(size_t)blockIdx.y * c + pj] = acc;
+}
+
+// y = s_C + the partial sums, chunks ascending.
+__global__ void y_kernel(ChainDev C, const double *part, int chunks, double *y) {
+  const int32_t c = C.c, pj = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x);
+  if (pj >= c) return;
+  double acc = C.s ? C.s[C.c_list[pj]] : 1.0 / (double)C.n;
+  for (int k = 0; k < chunks; ++k) acc += part[(size_t)k * c + pj];
+  y[pj] = acc;
+}
+
+// The triangular solves left after the elimination: CTA 0 L^T mu_C = z, CTA 1 U t = L^-1 P 1.
+__global__ void __launch_bounds__(1024, 1)
+chain_tail_kernel(const double *lu, int32_t c, const int32_t *piv, double *y, double *t) {
+  __shared__ TriScratch scratch;
+  if (blockIdx.x == 0) lower_t_solve(lu, c, piv, y, scratch);
+  else upper_solve(lu, c, t, scratch);
+}
+
+// mu, E[T] = sum mu, b_f = mu . f / E[T]; scalars[2] cleared for chain_rows_kernel.
+__global__ void __launch_bounds__(1024, 1)
+chain_total_kernel(ChainDev C, const double *y, double *mu, double *scalars) {
+  __shared__ double red[33];
+  const int32_t n = C.n;
+  const double unif = 1.0 / (double)n;
+  double part = 0.0, pf = 0.0;
   for (int32_t i = threadIdx.x; i < n; i += blockDim.x) {
     const int32_t pi = C.c_index[i];
-    const double m = pi >= 0 ? y[pi] : (C.s ? C.s[i] : 1.0 / (double)n);
+    const double m = pi >= 0 ? y[pi] : (C.s ? C.s[i] : unif);
     mu[i] = m;
     part += m;
+    if (C.f) pf = fma(m, C.f[i], pf);
+  }
+  const double T = block_sum(part, red);
+  if (C.f) pf = block_sum(pf, red);
+  if (threadIdx.x == 0) {
+    scalars[0] = T;
+    scalars[1] = C.f ? pf / T : 0.0;
+    scalars[2] = 0.0;
+    scalars[3] = (double)C.c;
+  }
+}
+
+// b = mu / E[T], and max_i (N 1)_i: t on C, 1 + sum_j Q_ij t_j on the other rows (a warp per row);
+// the maximum of positive doubles as an integer maximum of their bits.
+__global__ void __launch_bounds__(256)
+chain_rows_kernel(ChainDev C, const double *t, const int32_t *nzptr, const int32_t *nzcol,
+                  const double *nzval, const double *mu, double *b, double *scalars) {
+  const int32_t n = C.n, c = C.c;
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+  const double T = scalars[0];
+  for (int32_t i = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x); i < n;
+       i += (int32_t)(gridDim.x * blockDim.x))
+    b[i] = mu[i] / T;
+  unsigned long long best = 0ull;
+  for (int32_t i = (int32_t)warp; i < n; i += (int32_t)nwarps) {
+    const int32_t pi = C.c_index[i];
     double ti;
     if (pi >= 0) {
       ti = t[pi];
     } else {
-      ti = 1.0;
-      for (int32_t e = nzptr[i]; e < nzptr[i + 1]; ++e)
-        if (nzcol[e] < c) ti += nzval[e] * t[nzcol[e]];
+      double acc = 0.0;
+      for (int32_t e = nzptr[i] + (int32_t)lane; e < nzptr[i + 1]; e += 32) {
+        const int32_t pj = nzcol[e];
+        if (pj < c) acc = fma(nzval[e], t[pj], acc);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
+      ti = 1.0 + acc;
     }
-    tmax = fmax(tmax, ti);
+    const unsigned long long bits = ti > 0.0 ? (unsigned long long)__double_as_longlong(ti) : 0ull;
+    best = bits > best ? bits : best;
   }
-  const double T = block_sum(part, red);
-  tmax = block_max(tmax, red);
-  double bf = 0.0;
-  for (int32_t i = threadIdx.x; i < n; i += blockDim.x) {
-    const double bi = mu[i] / T;
-    b[i] = bi;
-    if (C.f) bf += bi * C.f[i];
-  }
-  bf = block_sum(bf, red);
-  if (threadIdx.x == 0) {
-    scalars[0] = T;
-    scalars[1] = C.f ? bf : 0.0;
-    scalars[2] = tmax;
-    scalars[3] = (double)c;
-  }
-  (void)rowscale;
+  if (lane == 0 && best) atomicMax(reinterpret_cast<unsigned long long *>(&scalars[2]), best);
 }
 
 cudaError_t launch_solve(const ChainDev &C, double *mu, double *b, double *scalars, double *lu,
                          int32_t *piv, unsigned char *ws, const SolveWs &L, uint32_t *status_dev,
-                         cudaStream_t stream) {
+                         int smem_optin, cudaStream_t stream) {
   const int32_t n = C.n, c = C.c;
   double *y = reinterpret_cast<double *>(ws + L.off_y);
   double *t = reinterpret_cast<double *>(ws + L.off_t);
@@ -277,17 +329,23 @@ cudaError_t launch_solve(const ChainDev &C, double *mu, double *b, double *scala
   int32_t *nzcol = reinterpret_cast<int32_t *>(ws + L.off_nzcol);
   double *nzval = reinterpret_cast<double *>(ws + L.off_nzval);
   int32_t *nnz_row = reinterpret_cast<int32_t *>(ws + L.off_flags);
+  double *part = reinterpret_cast<double *>(ws + L.off_slab);   // a slab holds n (c + 1) doubles
   const int64_t want_blocks = ((int64_t)n * 32 + 255) / 256;
   const int blocks = (int)(want_blocks < 2048 ? want_blocks : 2048);
-  const int64_t want_id = ((int64_t)c * c + 255) / 256;
-  const int id_blocks = (int)(want_id < 4096 ? want_id : 4096);
   row_prep_kernel<<<blocks, 256, 0, stream>>>(C, rowscale, nnz_row);
   exclusive_scan_kernel<<<1, 1024, 0, stream>>>(n, nnz_row, nzptr);
-  if (c > 0) identity_kernel<<<id_blocks, 256, 0, stream>>>(lu, c);
-  cudaMemsetAsync(y, 0, sizeof(double) * (size_t)(c > 0 ? c : 1), stream);
-  row_fill_kernel<<<blocks, 256, 0, stream>>>(C, rowscale, nzptr, nzcol, nzval, lu, y);
-  chain_solve_kernel<<<1, 1024, 0, stream>>>(C, lu, piv, y, t, rowscale, nzptr, nzcol, nzval, mu,
-                                             b, scalars, status_dev);
+  row_fill_kernel<<<blocks, 256, 0, stream>>>(C, rowscale, nzptr, nzcol, nzval, lu, t);
+  if (c > 0) {
+    const int chunks = std::min(n, 64);
+    u_rows_kernel<<<dim3((unsigned)((c + 127) / 128), (unsigned)chunks), 128, 0, stream>>>(C, rowscale, part);
+    y_kernel<<<(c + 127) / 128, 128, 0, stream>>>(C, part, chunks, y);
+    const LuBatch B{lu, 0, piv, 0, y, t, nullptr, status_dev};
+    cudaError_t e = launch_lu(B, c, 1, smem_optin, stream);
+    if (e != cudaSuccess) return e;
+    chain_tail_kernel<<<2, 1024, 0, stream>>>(lu, c, piv, y, t);
+  }
+  chain_total_kernel<<<1, 1024, 0, stream>>>(C, y, mu, scalars);
+  chain_rows_kernel<<<blocks, 256, 0, stream>>>(C, t, nzptr, nzcol, nzval, mu, b, scalars);
   return cudaGetLastError();
 }
 

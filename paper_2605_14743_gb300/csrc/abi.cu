@@ -198,7 +198,9 @@ McDev to_dev(const afc_mc_problem &p, uint32_t r_begin, uint32_t *counts, afc_mc
 // the other warps help with the per-realization steps only) and grid.
 struct McPlan {
   int block = 1024;
+  bool chip = false;   // the kernel's on-chip form for small graphs
   uint32_t nsw = 1, smem = 0, grid = 1;
+  uint32_t slots = 0;      // compact source slots that shared memory holds
   bool fits = true;
 };
 
@@ -207,6 +209,14 @@ struct McPlan {
 uint32_t slots_within(uint32_t n, uint64_t arcs, uint32_t bytes) {
   return mc_slots_within(n, arcs, bytes);
 }
+
+// Graphs of up to this many nodes run the counting kernel's on-chip form.  Their time goes into the
+// serial phases of each realization and into settle steps with few nodes, so several CTAs share an
+// SM (1024 threads together), each as small as still fills the GPU with the call's realizations:
+// few realizations take more warps each.  Measured (ms a call, on-chip form / 1024-thread CTAs
+// with the scratch in device memory; 4,096 realizations, ER of mean degree 6): n = 50 2.29 / 3.56,
+// 80 4.62 / 6.16, 120 8.23 / 9.58, 200 19.5 / 20.4, 300 38.9 / 38.5, 450 96.9 / 75.4.
+constexpr uint32_t kSmallNodes = 240;
 
 // want_warps: source warps the launch should offer (0: as many as fit for the largest graph;
 // a batched launch passes the most that any of its problems can use).
@@ -217,8 +227,14 @@ McPlan plan_for(const afc_mc_problem &p0, uint32_t nmax, uint64_t amax, uint64_t
   const uint32_t cap = (uint32_t)std::max(0, d.smem_optin - 1024);
   // node ids share their 16-bit settle-order entries with a step mark: below 2^15 nodes
   const uint32_t fit = nmax < 32768u ? slots_within(nmax, amax, cap) : 0u;
+  pl.slots = fit;
+  pl.chip = nmax <= kSmallNodes &&
+            mc_layout_bytes(nmax, amax, std::min<uint32_t>(fit, 32u), true) <= cap;
   if (p0.block_threads) {
     pl.block = p0.block_threads;
+  } else if (pl.chip) {
+    const uint64_t warps = (uint64_t)std::max(1, d.sms) * (kSmallThreadsPerSm / 32);
+    pl.block = total_items * 8u >= warps ? 256 : total_items * 16u >= warps ? 512 : 1024;
   } else {
     // the smallest CTA that holds a warp for every slot that fits (fewer threads per CTA leave
     // each thread more registers for the source warps' caches)
@@ -228,10 +244,11 @@ McPlan plan_for(const afc_mc_problem &p0, uint32_t nmax, uint64_t amax, uint64_t
   pl.nsw = std::min<uint32_t>(fit, (uint32_t)pl.block / 32u);
   pl.fits = pl.nsw >= 1;
   if (pl.fits) {
-    pl.smem = mc_layout_bytes(nmax, amax, pl.nsw);
+    pl.smem = mc_layout_bytes(nmax, amax, pl.nsw, pl.chip);
     const uint32_t smem_sm = 228u * 1024u;
-    const uint32_t per_sm = std::max<uint32_t>(1u, std::min<uint32_t>(smem_sm / (pl.smem + 1024u),
-                                                                      2048u / (uint32_t)pl.block));
+    const uint32_t threads = pl.chip ? (uint32_t)kSmallThreadsPerSm : 2048u;
+    const uint32_t per_sm = std::max<uint32_t>(
+        1u, std::min<uint32_t>(smem_sm / (pl.smem + 1024u), threads / (uint32_t)pl.block));
     pl.grid = (uint32_t)std::min<uint64_t>(total_items, (uint64_t)d.sms * per_sm);
   }
   if (pl.grid == 0) pl.grid = 1;
@@ -389,7 +406,7 @@ bool wants_global(const afc_mc_problem &p) {
   if (p.memory_path == AFC_PATH_GLOBAL) return true;
   if (p.memory_path == AFC_PATH_SHARED) return false;
   const McPlan pl = plan_for(p, (uint32_t)p.n, 2ull * (uint64_t)p.m, 1);
-  return !pl.fits || pl.nsw < kMinSharedSlots;
+  return !pl.fits || std::min(pl.slots, p.block_threads ? pl.nsw : 32u) < kMinSharedSlots;
 }
 
 size_t meta_bytes(int nprob) {
@@ -414,6 +431,13 @@ SharedBatch shared_batch(int nprob, const afc_mc_problem *probs, const uint32_t 
   for (int g = 0; g < nprob; ++g)
     if (!wants_global(probs[g])) sb.order.push_back(g);
   if (sb.order.empty()) return sb;
+  // the costliest realizations first: the CTAs claim items in this order, so the launch ends on
+  // small ones (8 graphs of 230-1,730 nodes, 96 realizations each: 95 -> 84 ms a call; 12 of
+  // 230-1,180, 115 each: 73 -> 60)
+  std::stable_sort(sb.order.begin(), sb.order.end(), [&](int a, int b) {
+    auto per = [&](int g) { return (double)probs[g].n * (double)(probs[g].n + 2 * probs[g].m); };
+    return per(a) > per(b);
+  });
   const DevInfo di = dev_info();
   const uint32_t cap = (uint32_t)std::max(0, di.smem_optin - 1024);
   double work = 0.0, small_work = 0.0, long_work = 0.0;
@@ -510,13 +534,14 @@ int run_counts(int nprob, const afc_mc_problem *probs, const uint32_t *r_begin,
       for (int k = 0; k < ns; ++k) {
         const afc_mc_problem &p = probs[order[k]];
         const uint32_t fit = slots_within((uint32_t)p.n, 2ull * (uint64_t)p.m, pl.smem);
-        devs[k].spt = std::max<uint32_t>(1u, std::min<uint32_t>(fit, (uint32_t)pl.block / 32u));
+        devs[k].spt = pl.chip ? pl.nsw
+                              : std::max<uint32_t>(1u, std::min<uint32_t>(fit, (uint32_t)pl.block / 32u));
       }
       AFC_CUDA(cudaMemcpyAsync(devs_d, devs.data(), sizeof(McDev) * (size_t)ns, cudaMemcpyHostToDevice, stream));
     }
     // the shared batch's grid was sized for all its items: the launch may use fewer CTAs
     const uint32_t grid = (uint32_t)std::min<uint64_t>(pl.grid, prefix[ns]);
-    cudaError_t e = launch_mc_counts(pl.block, sb.long_form, devs_d, ns, prefix_d, prefix[ns], pl.nsw, pl.smem,
+    cudaError_t e = launch_mc_counts(pl.block, sb.long_form, pl.chip, devs_d, ns, prefix_d, prefix[ns], pl.nsw, pl.smem,
                                      std::max<uint32_t>(grid, 1u), ws + meta_bytes(nprob),
                                      sb.scratch_stride, stream);
     if (e != cudaSuccess) return cuda_fail(e, "counting kernel launch");
@@ -794,7 +819,7 @@ int afc_debug_components(const afc_mc_problem *prob, uint32_t r_begin, uint32_t 
   if (st) return st;
   if (!comp || !csize) return fail(AFC_EINVAL, "null output");
   const DevInfo di = dev_info();
-  if ((int)mc_layout_bytes(prob->n, 2 * prob->m, 0) > di.smem_optin)
+  if ((int)mc_layout_bytes(prob->n, 2 * prob->m, 0, false) > di.smem_optin)
     return fail(AFC_EUNSUPPORTED, "graph too large for the shared-memory component kernel");
   if (r_count == 0) return AFC_OK;
   McDev d = to_dev(*prob, r_begin, nullptr, nullptr, nullptr, nullptr);

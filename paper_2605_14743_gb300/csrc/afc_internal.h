@@ -52,7 +52,9 @@ afc_host_query host_query_of(const afc_graph *g, const afc_params *p, uint32_t n
 // mc_kernel.cu: the shared-memory path (one warp per source, settle steps)
 // Shared memory of a counting CTA of the shared-memory path: a graph of n nodes and `arcs`
 // arcs, and `nsw` warps that each own one source slot.
-uint32_t mc_layout_bytes(uint32_t n, uint64_t arcs, uint32_t nsw);
+uint32_t mc_layout_bytes(uint32_t n, uint64_t arcs, uint32_t nsw, bool chip);
+// Threads per SM of the on-chip form's CTAs (64 registers each).
+constexpr int kSmallThreadsPerSm = 1024;
 // Compact source slots that fit next to the realization within `bytes` (0 unless at least one
 // wide slot fits).
 uint32_t mc_slots_within(uint32_t n, uint64_t arcs, uint32_t bytes);
@@ -60,8 +62,9 @@ uint32_t mc_slots_within(uint32_t n, uint64_t arcs, uint32_t bytes);
 // components, source list, selection scratch and betweenness accumulators.
 size_t mc_cta_scratch_bytes(uint32_t n);
 // long_form: the LONG form of the source routine (StepGraph in mc_steps.cuh)
-cudaError_t launch_mc_counts(int block, bool long_form, const McDev *probs_dev, int nprob,
-                             const uint64_t *prefix_dev, uint64_t total_items,
+// chip: the on-chip form for small graphs
+cudaError_t launch_mc_counts(int block, bool long_form, bool chip, const McDev *probs_dev, int nprob,
+                             uint64_t *prefix_dev, uint64_t total_items,
                              uint32_t source_warps, uint32_t smem_bytes, uint32_t grid,
                              unsigned char *scratch, size_t scratch_stride, cudaStream_t stream);
 cudaError_t launch_debug_realize(const McDev &P, uint32_t r_count, uint8_t *alive, uint32_t *w,

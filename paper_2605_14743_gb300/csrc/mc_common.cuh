@@ -254,14 +254,16 @@ __device__ __forceinline__ void fx_red(unsigned long long *a0, unsigned long lon
   if (f0) atomicAdd(&a2[v], (unsigned long long)f0);
 }
 
-// B_v as a double, written over a0 (each thread converts its own entries).
+// B_v as a double, written to out, by default over a0 (each thread converts its own entries).
 __device__ __forceinline__ void fx_finalize3(unsigned long long *a0, const unsigned long long *a1,
-                                             const unsigned long long *a2, uint32_t n) {
+                                             const unsigned long long *a2, uint32_t n,
+                                             double *out = nullptr) {
+  if (!out) out = reinterpret_cast<double *>(a0);
   for (uint32_t v = threadIdx.x; v < n; v += blockDim.x) {
     const unsigned long long t = a1[v];
     const unsigned long long lo = a2[v] + (t << 32);
     const unsigned long long hi = a0[v] + (t >> 32) + (lo < (t << 32) ? 1ull : 0ull);
-    reinterpret_cast<double *>(a0)[v] = (double)hi + __ull2double_rn(lo) * 0x1p-64;
+    out[v] = (double)hi + __ull2double_rn(lo) * 0x1p-64;
   }
 }
 
@@ -857,6 +859,59 @@ __device__ inline void realize_csr(const McDev &P, uint32_t r, uint32_t *rp, uin
   if ((threadIdx.x & 31u) == 0) atomicMax(&ctl->wmax, wmax);
   const uint32_t total = ctl->scan_total;
   if (threadIdx.x == 0) rp[n] = total < cap ? total : cap;
+  __syncthreads();
+}
+
+// realize_csr for a realization built on chip: each arc is drawn once (an arc per thread, or a
+// node's arcs per thread in the hop mode) into tmp [2 m] (shared memory), then compacted.  Small
+// graphs spend most of their time in such per-realization phases.
+__device__ inline void realize_csr_chip(const McDev &P, uint32_t r, uint32_t *rp, uint32_t *arc,
+                                        uint32_t *tmp, CtaHead *ctl, const uint32_t *hop) {
+  constexpr uint32_t kDead = 0xFFFFFFFFu;   // no alive arc: length 65535 to node 65535 >= n
+  const uint32_t n = P.n, arcs = (uint32_t)(2 * P.m), T = blockDim.x;
+  uint32_t wmax = 1, err = 0;
+  auto draw = [&](uint32_t a) -> uint32_t {
+    const uint32_t e = (uint32_t)P.eid[a], u = (uint32_t)P.col[a];
+    if (e >= (uint64_t)P.m || u >= n) { err = kErrInput; return kDead; }
+    bool alive; uint32_t w;
+    edge_draw(P, r, e, alive, w);
+    if (!alive) return kDead;
+    if (w == 0 || w > 0xFFFFu) { err = kErrInput; return kDead; }
+    wmax = max(wmax, w);
+    return u | (w << 16);
+  };
+  if (hop) {
+    for (uint32_t v = threadIdx.x; v < n; v += T)
+      for (int32_t a = P.row_ptr[v]; a < P.row_ptr[v + 1]; ++a) {
+        if (a < 0 || (uint32_t)a >= arcs) { err = kErrInput; continue; }
+        const uint32_t u = (uint32_t)P.col[a];
+        tmp[a] = hop[v] > P.hop_radius || u >= n || hop[u] > P.hop_radius ? kDead : draw((uint32_t)a);
+      }
+  } else {
+    for (uint32_t a = threadIdx.x; a < arcs; a += T) tmp[a] = draw(a);
+  }
+  __syncthreads();
+  const uint32_t per = (n + T - 1) / T;
+  const uint32_t v0 = min(n, threadIdx.x * per), v1 = min(n, v0 + per);
+  auto each = [&](uint32_t v, auto &&f) {
+    const int32_t a0 = max(P.row_ptr[v], 0), a1 = min(P.row_ptr[v + 1], (int32_t)arcs);
+    for (int32_t a = a0; a < a1; ++a)
+      if (tmp[a] != kDead) f(tmp[a]);
+  };
+  uint32_t cnt = 0;
+  for (uint32_t v = v0; v < v1; ++v) each(v, [&](uint32_t) { ++cnt; });
+  uint32_t off = block_exclusive_scan(cnt, ctl->scan, &ctl->scan_total);
+  for (uint32_t v = v0; v < v1; ++v) {
+    rp[v] = min(off, arcs);
+    each(v, [&](uint32_t x) {
+      if (off < arcs) arc[off++] = x; else err = kErrInput;
+    });
+  }
+  if (err) atomicOr(&ctl->err, err);
+  wmax = __reduce_max_sync(kFull, wmax);
+  if ((threadIdx.x & 31u) == 0) atomicMax(&ctl->wmax, wmax);
+  const uint32_t total = ctl->scan_total;
+  if (threadIdx.x == 0) rp[n] = total < arcs ? total : arcs;
   __syncthreads();
 }
 

@@ -30,10 +30,10 @@ namespace afc {
 // wide_slots() 16-byte slots for a realization with a length above kCompactMaxLen or a path
 // count above 2^32 - 1; it is never smaller than one wide slot.
 struct StepLayout {
-  uint32_t off_rp, off_arc, off_mw, off_slots;
+  uint32_t off_rp, off_arc, off_mw, off_slots, off_chip;
   uint32_t slot_bytes, wide_bytes, total;
   __host__ __device__ static uint32_t al(uint32_t x) { return al16(x); }
-  __host__ __device__ void make(uint32_t n, uint32_t arcs, uint32_t nsw) {
+  __host__ __device__ void make(uint32_t n, uint32_t arcs, uint32_t nsw, bool chip = false) {
     uint32_t o = al(sizeof(CtaHead));
     off_rp = o;     o = al(o + 2u * (n + 1));
     off_arc = o;    o = al(o + 4u * (arcs > 0 ? arcs : 1));
@@ -42,7 +42,13 @@ struct StepLayout {
     slot_bytes = al(4u * n) + al(8u * n);
     wide_bytes = slot_bytes + 2u * al(2u * n);
     const uint32_t region = nsw * slot_bytes;
-    total = o + (nsw == 0 ? 0u : (region > wide_bytes ? region : wide_bytes));
+    off_chip = o + (nsw == 0 ? 0u : (region > wide_bytes ? region : wide_bytes));
+    total = off_chip + (chip ? chip_bytes(n, arcs) : 0u);
+  }
+  // on-chip form (small graphs): comp, cinfo, sel, src, the betweenness as doubles and the drawn
+  // arcs, after the slots
+  __host__ __device__ static uint32_t chip_bytes(uint32_t n, uint32_t arcs) {
+    return 3u * al(4u * n) + al(2u * n) + al(8u * n) + al(4u * (arcs > 0 ? arcs : 1));
   }
   // wide slots in the region of nsw compact ones (at least one)
   __host__ __device__ uint32_t wide_slots(uint32_t nsw) const {
@@ -84,40 +90,56 @@ struct CtaScratch {
 };
 
 // ---------------------------------------------------------------------------------------
-// The persistent kernel.  Work item w enumerates (problem, realization) pairs of all
-// problems; items are visited in strided order by the CTAs.  Inside a realization the source
-// warps claim sources one at a time.
+// The persistent kernel.  Work item w enumerates (problem, realization) pairs of all problems,
+// the costliest realizations first; each CTA starts with the item of its index and claims the next
+// ones from a counter (item_prefix[0], 0 at the launch: the prefix of the first problem is 0), so
+// that the last CTAs to finish do so on small items.  Inside a realization the source warps claim
+// sources one at a time.
 // ---------------------------------------------------------------------------------------
-template <int BLOCK, bool LONG>
-__global__ void __launch_bounds__(BLOCK, 1)
-mc_counts_kernel(const McDev *__restrict__ probs, int nprob, const uint64_t *item_prefix,
+//
+// CHIP (small graphs): components, source list, selection scratch and the drawn arcs also live in
+// shared memory, and several CTAs of few warps share an SM (64 registers a thread), so that one
+// realization's serial phases overlap the others'.
+template <int BLOCK, bool LONG, bool CHIP>
+__global__ void __launch_bounds__(BLOCK, CHIP ? kSmallThreadsPerSm / BLOCK : 1)
+mc_counts_kernel(const McDev *__restrict__ probs, int nprob, uint64_t *item_prefix,
                  uint64_t total_items, uint32_t nsw_launch, unsigned char *scratch,
                  size_t scratch_stride) {
   extern __shared__ __align__(16) unsigned char smem[];
   CtaHead *ctl = reinterpret_cast<CtaHead *>(smem);
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
   unsigned char *const my_scratch = scratch + (size_t)blockIdx.x * scratch_stride;
-  for (uint64_t item = blockIdx.x; item < total_items; item += gridDim.x) {
+  for (uint64_t item = blockIdx.x; item < total_items; item = ctl->next_item) {
     int g = 0;
     while (g + 1 < nprob && item_prefix[g + 1] <= item) ++g;
     const McDev &P = probs[g];
     // source warps: per problem in a batched launch (small graphs use more of the CTA's
     // warps), else the launch's value
     const uint32_t nsw = P.spt ? P.spt : nsw_launch;
-    const uint32_t r_local = (uint32_t)(item - item_prefix[g]);
+    const uint32_t r_local = (uint32_t)(item - (g ? item_prefix[g] : 0u));
     uint32_t anchor;
     const uint32_t r = item_rho(P, r_local, anchor);
     const uint32_t n = P.n;
     StepLayout L;
-    L.make(n, (uint32_t)(2 * P.m), nsw);
+    L.make(n, (uint32_t)(2 * P.m), nsw, CHIP);
     uint16_t *rp16 = reinterpret_cast<uint16_t *>(smem + L.off_rp);
     uint32_t *rp = reinterpret_cast<uint32_t *>(smem + L.off_slots);   // until the sources run
     uint32_t *arc = reinterpret_cast<uint32_t *>(smem + L.off_arc);
     uint32_t *mwt = reinterpret_cast<uint32_t *>(smem + L.off_mw);
     CtaScratch cs;
     cs.carve(my_scratch, n);
-    uint32_t *comp = cs.comp, *cinfo = cs.cinfo, *sel = cs.sel;
+    uint32_t *comp = cs.comp, *cinfo = cs.cinfo, *sel = cs.sel, *drawn = nullptr;
     uint16_t *src = cs.src;
+    double *bc = reinterpret_cast<double *>(cs.a0);
+    if constexpr (CHIP) {
+      unsigned char *q = smem + L.off_chip;
+      comp = reinterpret_cast<uint32_t *>(q);   q += StepLayout::al(4u * n);
+      cinfo = reinterpret_cast<uint32_t *>(q);  q += StepLayout::al(4u * n);
+      sel = reinterpret_cast<uint32_t *>(q);    q += StepLayout::al(4u * n);
+      src = reinterpret_cast<uint16_t *>(q);    q += StepLayout::al(2u * n);
+      bc = reinterpret_cast<double *>(q);       q += StepLayout::al(8u * n);
+      drawn = reinterpret_cast<uint32_t *>(q);
+    }
     if (threadIdx.x == 0) {
       ctl->err = 0; ctl->ovf = 0; ctl->nsrc = 0; ctl->cursor = 0; ctl->wide_redo = 0;
       ctl->edges = 0; ctl->verts = 0; ctl->wmax = 1;
@@ -126,7 +148,8 @@ mc_counts_kernel(const McDev *__restrict__ probs, int nprob, const uint64_t *ite
 
     const bool ball = P.per_row && P.hop_radius;
     if (ball) hop_ball(P, anchor, cinfo);   // cinfo is free until the components
-    realize_csr(P, r, rp, arc, ctl, ball ? cinfo : nullptr);
+    if constexpr (CHIP) realize_csr_chip(P, r, rp, arc, drawn, ctl, ball ? cinfo : nullptr);
+    else realize_csr(P, r, rp, arc, ctl, ball ? cinfo : nullptr);
     Realized H{n, rp, arc};
     components(P, H, comp, cinfo);
     if (P.per_row) keep_anchor_component(n, anchor, comp, cinfo);
@@ -229,14 +252,13 @@ mc_counts_kernel(const McDev *__restrict__ probs, int nprob, const uint64_t *ite
         if (threadIdx.x == 0 && P.stats) atomicAdd(u64p(&P.stats->wide_redone), 1ull);
         continue;
       }
-      fx_finalize3(cs.a0, cs.a1, cs.a2, n);   // betweenness as doubles, in a0's storage
+      fx_finalize3(cs.a0, cs.a1, cs.a2, n, bc);   // betweenness as doubles
       __syncthreads();
       SlotArrays scratch{};
       scratch.dist = s0.dist;
       scratch.sig = s0.sig;
       const bool recheck = select_and_count(P, r_local, comp, cinfo,
-                                            reinterpret_cast<const double *>(cs.a0), scratch, sel,
-                                            src, use32, ctl);
+                                            bc, scratch, sel, src, use32, ctl);
       __syncthreads();
       if (!recheck) break;
       use32 = false;
@@ -250,6 +272,7 @@ mc_counts_kernel(const McDev *__restrict__ probs, int nprob, const uint64_t *ite
       atomicAdd(u64p(&P.stats->vertex_visits), (unsigned long long)ctl->verts);
       if (ctl->ovf) atomicAdd(u64p(&P.stats->overflow), 1ull);
     }
+    if (threadIdx.x == 0) ctl->next_item = gridDim.x + atomicAdd(u64p(&item_prefix[0]), 1ull);
     __syncthreads();
   }
 }
@@ -354,9 +377,9 @@ debug_sssp_kernel(McDev P, uint32_t r, const int32_t *sources, int32_t nsrc, uin
 // ---------------------------------------------------------------------------------------
 // Host-side launch helpers (called from the C ABI)
 // ---------------------------------------------------------------------------------------
-uint32_t mc_layout_bytes(uint32_t n, uint64_t arcs, uint32_t nsw) {
+uint32_t mc_layout_bytes(uint32_t n, uint64_t arcs, uint32_t nsw, bool chip) {
   StepLayout L;
-  L.make(n, (uint32_t)arcs, nsw);
+  L.make(n, (uint32_t)arcs, nsw, chip);
   return L.total;
 }
 
@@ -372,32 +395,31 @@ size_t mc_cta_scratch_bytes(uint32_t n) { return CtaScratch::bytes(n); }
 
 #define AFC_MC_BLOCKS(X) X(256) X(512) X(1024)
 
-template <int BLOCK, bool LONG>
-static cudaError_t launch_counts_t(const McDev *probs_dev, int nprob, const uint64_t *prefix_dev,
+template <int BLOCK, bool LONG, bool CHIP>
+static cudaError_t launch_counts_t(const McDev *probs_dev, int nprob, uint64_t *prefix_dev,
                                    uint64_t total_items, uint32_t nsw, uint32_t smem,
                                    uint32_t grid, unsigned char *scratch, size_t stride,
                                    cudaStream_t stream) {
-  cudaFuncSetAttribute(mc_counts_kernel<BLOCK, LONG>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  mc_counts_kernel<BLOCK, LONG><<<grid, BLOCK, smem, stream>>>(probs_dev, nprob, prefix_dev,
-                                                               total_items, nsw, scratch, stride);
+  cudaFuncSetAttribute(mc_counts_kernel<BLOCK, LONG, CHIP>,
+                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  mc_counts_kernel<BLOCK, LONG, CHIP><<<grid, BLOCK, smem, stream>>>(
+      probs_dev, nprob, prefix_dev, total_items, nsw, scratch, stride);
   return cudaGetLastError();
 }
 
-cudaError_t launch_mc_counts(int block, bool long_form, const McDev *probs_dev, int nprob,
-                             const uint64_t *prefix_dev, uint64_t total_items,
+cudaError_t launch_mc_counts(int block, bool long_form, bool chip, const McDev *probs_dev,
+                             int nprob, uint64_t *prefix_dev, uint64_t total_items,
                              uint32_t source_warps, uint32_t smem_bytes, uint32_t grid,
                              unsigned char *scratch, size_t scratch_stride, cudaStream_t stream) {
   if (source_warps < 1 || source_warps > (uint32_t)block / 32u) return cudaErrorInvalidValue;
-#define AFC_X(B)                                                                             \
-  if (block == B)                                                                            \
-    return long_form                                                                         \
-               ? launch_counts_t<B, true>(probs_dev, nprob, prefix_dev, total_items,         \
-                                          source_warps, smem_bytes, grid, scratch,           \
-                                          scratch_stride, stream)                            \
-               : launch_counts_t<B, false>(probs_dev, nprob, prefix_dev, total_items,        \
-                                           source_warps, smem_bytes, grid, scratch,          \
-                                           scratch_stride, stream);
-  AFC_MC_BLOCKS(AFC_X)
+#define AFC_X(B, LG, CH)                                                                  \
+  if (block == B && long_form == LG && chip == CH)                                        \
+    return launch_counts_t<B, LG, CH>(probs_dev, nprob, prefix_dev, total_items,          \
+                                      source_warps, smem_bytes, grid, scratch,            \
+                                      scratch_stride, stream);
+#define AFC_XB(B) AFC_X(B, false, false) AFC_X(B, true, false) AFC_X(B, false, true) AFC_X(B, true, true)
+  AFC_MC_BLOCKS(AFC_XB)
+#undef AFC_XB
 #undef AFC_X
   return cudaErrorInvalidValue;
 }

@@ -86,7 +86,7 @@ struct WarpScratch {
 // Control fields of a CTA that works on one realization (realization, components, selection).
 struct CtaHead {
   uint32_t err, ovf, nsrc, cursor;
-  unsigned long long edges, verts;
+  unsigned long long edges, verts, next_item;
   uint32_t need_recheck, delta, dsh, wmax;
   uint32_t scan[32];
   uint32_t scan_total, wide_redo, pad2, pad3;   // wide_redo: a path count needs 64-bit slots

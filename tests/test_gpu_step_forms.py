@@ -70,3 +70,31 @@ def test_stars_and_single_arcs():
     for w_lo in (1, 100):
         for path in (SHARED, GLOBAL):
             _check(Workload("star", n, eu, ev, 0.95, w_lo, 100, 2, seed=2, k_min=2), 2, path)
+
+
+@pytest.mark.parametrize("n,R", [(1, 3), (2, 3), (33, 700), (240, 4), (241, 4)])
+@pytest.mark.parametrize("w_hi", [9, 50])
+def test_small_graph_form(n, R, w_hi):
+    """The on-chip form's range (240 nodes), its smallest graphs, and more realizations than CTAs
+    (the others are claimed); few realizations take CTAs of more warps."""
+    eu, ev = ws_edges(n, 4, 0.2, 6) if n > 4 else path_edges(n)
+    _check(Workload("small", n, eu, ev, 0.85, 1, w_hi, R, seed=8, k_min=2), R, SHARED)
+
+
+def test_small_dense_graph_without_room_for_the_drawn_arcs():
+    """A complete graph of 170 nodes: its arcs fit on chip once, not twice."""
+    from afc_inputs import complete_edges
+    eu, ev = complete_edges(170)
+    _check(Workload("dense", 170, eu, ev, 0.5, 1, 40, 2, seed=4), 2, SHARED)
+
+
+@pytest.mark.parametrize("block", [256, 512, 1024])
+def test_small_graph_block_sizes(block):
+    eu, ev = er_edges(60, 0.1, 3)
+    wl = Workload("blocks", 60, eu, ev, 0.9, 1, 10, 40, seed=2)
+    a = afc.Query(wl, block_threads=block)
+    b = afc.Query(wl, memory_path=GLOBAL)
+    a.run_counts()
+    b.run_counts()
+    torch.cuda.synchronize()
+    assert (a.counts == b.counts).all() and (a.stats[:3] == b.stats[:3]).all()

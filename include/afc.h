@@ -506,8 +506,8 @@ typedef struct {
   uint64_t *solve_stats;     /* [2] DEVICE or NULL, accumulated: perturbations whose reduced  */
                              /* systems were solved by defect correction on the nominal     */
                              /* factors, and by factoring I - Q'_CC (large c only: c x c     */
-                             /* matrices that do not fit in shared memory; small c always   */
-                             /* factors in shared memory and counts neither)                 */
+                             /* matrices that do not fit in shared memory; small c counts    */
+                             /* neither)                                                     */
 } afc_perturb_params;
 
 /* DEVICE outputs (accumulated, caller zeroes): counters [3] = {top-1 changes, top-k set

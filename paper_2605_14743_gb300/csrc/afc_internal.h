@@ -89,13 +89,12 @@ struct ChainDev {
 
 // Workspace carve-up of the solve path (byte offsets), shared by solve and perturb.
 struct SolveWs {
-  size_t off_y, off_t, off_rowscale, off_nzptr, off_nzcol, off_nzval, off_flags, off_tmp, off_csc,
+  size_t off_y, off_t, off_rowscale, off_nzptr, off_nzcol, off_nzval, off_flags, off_tmp, off_inv,
       off_slab, total;
   size_t nnz_cap;
-  size_t csc_cap;   // entries of the column-wise pattern of Q_CC the large-c sweep builds (0: none)
 };
 SolveWs solve_ws_layout(int32_t n, int32_t c, size_t nnz_cap, uint32_t perturb_slabs,
-                        size_t slab_bytes, size_t csc_cap);
+                        size_t slab_bytes, size_t inverse_bytes);
 
 cudaError_t launch_observed_states(int32_t n, const uint32_t *counts, int32_t *c_index,
                                    int32_t *c_list, int32_t *c_dev, cudaStream_t stream);
@@ -111,8 +110,13 @@ cudaError_t launch_certificates(const ChainDev &C, const double *mu0, const doub
                                 const int32_t *piv0, double eps_bar, double r_min, int32_t npairs,
                                 const int32_t *pu, const int32_t *pv, double *gap, double *sharp,
                                 unsigned char *ws, const SolveWs &L, cudaStream_t stream);
+// The right-hand side y0 = s_C + s_U Q_UC of the reduced solve (part: 64 c doubles of scratch).
+void launch_nominal_rhs(const ChainDev &C, const double *rowscale, double *part, double *y,
+                        cudaStream_t stream);
+// Device memory of one sweep CTA, and of the nominal matrix's FP32 inverse and its transpose.
 size_t perturb_slab_bytes(int32_t n, int32_t c);
-// true when the sweep keeps a perturbation's c x c matrix in shared memory (else: device slabs)
+size_t perturb_inverse_bytes(int32_t c);
+// true when the sweep factors a perturbation's c x c matrix in shared memory (else: device slabs)
 bool perturb_on_chip(int32_t c, int smem_optin);
 // bootstrap.cu: realization-level bootstrap replicates of b and their percentile intervals
 size_t bootstrap_slab_bytes(int32_t n, int32_t c, uint32_t R);
@@ -195,6 +199,5 @@ cudaError_t launch_solve_static(int32_t n, uint32_t R, double alpha, double eta,
                                 double *scalars, uint32_t *status_host, int32_t *c_host,
                                 cudaStream_t stream);
 size_t solve_static_bytes();
-uint32_t perturb_smem_bytes(int32_t n, int32_t c);
 
 }  // namespace afc

@@ -81,7 +81,7 @@ cudaError_t launch_observed_states(int32_t n, const uint32_t *counts, int32_t *c
 
 // ---- workspace ----------------------------------------------------------------------------
 SolveWs solve_ws_layout(int32_t n, int32_t c, size_t nnz_cap, uint32_t perturb_slabs,
-                        size_t slab_bytes, size_t csc_cap) {
+                        size_t slab_bytes, size_t inverse_bytes) {
   auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
   SolveWs L{};
   size_t o = 0;
@@ -94,8 +94,7 @@ SolveWs solve_ws_layout(int32_t n, int32_t c, size_t nnz_cap, uint32_t perturb_s
   L.off_nzval = o;    o = al(o + 8 * nnz_cap);
   L.off_flags = o;    o = al(o + 4 * (size_t)n + 64);
   L.off_tmp = o;      o = al(o + 8 * (4 * (size_t)n + 4 * cc + 64));
-  L.off_csc = o;      o = al(o + (csc_cap ? 4 * ((cc + 1 + 63) & ~size_t(63)) + 8 * csc_cap : 0));
-  L.csc_cap = csc_cap;
+  L.off_inv = o;      o = al(o + inverse_bytes);
   L.off_slab = o;     o = al(o + (size_t)perturb_slabs * slab_bytes);
   L.total = o;
   L.nnz_cap = nnz_cap;
@@ -318,6 +317,15 @@ chain_rows_kernel(ChainDev C, const double *t, const int32_t *nzptr, const int32
   if (lane == 0 && best) atomicMax(reinterpret_cast<unsigned long long *>(&scalars[2]), best);
 }
 
+void launch_nominal_rhs(const ChainDev &C, const double *rowscale, double *part, double *y,
+                        cudaStream_t stream) {
+  if (C.c <= 0) return;
+  const int chunks = std::min(C.n, 64);
+  const unsigned blocks = (unsigned)((C.c + 127) / 128);
+  u_rows_kernel<<<dim3(blocks, (unsigned)chunks), 128, 0, stream>>>(C, rowscale, part);
+  y_kernel<<<blocks, 128, 0, stream>>>(C, part, chunks, y);
+}
+
 cudaError_t launch_solve(const ChainDev &C, double *mu, double *b, double *scalars, double *lu,
                          int32_t *piv, unsigned char *ws, const SolveWs &L, uint32_t *status_dev,
                          int smem_optin, cudaStream_t stream) {
@@ -336,9 +344,7 @@ cudaError_t launch_solve(const ChainDev &C, double *mu, double *b, double *scala
   exclusive_scan_kernel<<<1, 1024, 0, stream>>>(n, nnz_row, nzptr);
   row_fill_kernel<<<blocks, 256, 0, stream>>>(C, rowscale, nzptr, nzcol, nzval, lu, t);
   if (c > 0) {
-    const int chunks = std::min(n, 64);
-    u_rows_kernel<<<dim3((unsigned)((c + 127) / 128), (unsigned)chunks), 128, 0, stream>>>(C, rowscale, part);
-    y_kernel<<<(c + 127) / 128, 128, 0, stream>>>(C, part, chunks, y);
+    launch_nominal_rhs(C, rowscale, part, y, stream);
     const LuBatch B{lu, 0, piv, 0, y, t, nullptr, status_dev};
     cudaError_t e = launch_lu(B, c, 1, smem_optin, stream);
     if (e != cudaSuccess) return e;

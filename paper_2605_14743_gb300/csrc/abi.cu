@@ -262,17 +262,20 @@ constexpr uint32_t kMinStepWarps = 4;
 
 // Whether the settle-step kernel outruns the bucketed one on this graph.  Its cost grows with
 // the range of lengths (a wider range settles fewer nodes per step against a pending list of
-// about the same length), the bucketed kernel's does not.  Measured on WS graphs of mean
-// degree 8 (k = 8, beta = 0.2, survival 0.9), lengths uniform in 1..W, realizations/s of the
-// settle-step kernel over the better bucketed team size: n = 2,500: W = 25 2.43x, 50 1.91x,
-// 100 1.51x, 400 1.29x; n = 3,200: 2.07x, 1.59x, 1.19x, 0.98x; n = 3,818: 1.89x, 1.45x, 1.07x,
-// 0.85x; n = 4,000: 1.73x, 1.31x, 0.96x, 0.75x; W = 100: n = 5,000 0.75x, 7,000 0.53x, 10,000
-// 0.30x.  The ratio goes about as n^-1.17 and min(W, 200)^-0.35, which puts the crossover at
-// n min(W, 200)^0.35 = 19,500 (n = 6,400 for W = 25, 5,000 for W = 50, 3,900 for W = 100,
-// 3,050 for W >= 200).  Per-edge length ranges and length laws count as W = 65,535.
+// about the same length), the bucketed kernel's does not; and with n it runs out of warps, each
+// of which keeps a distance array on chip (8 warps per CTA at n = 7,200, 5 at 10,500).  Measured
+// on graphs of mean degree 8 (survival 0.9), lengths uniform in 1..W, ms of the bucketed kernel
+// over ms of the settle-step kernel, WS k = 8 beta = 0.1 / ER: n = 2,700: W = 100 1.62 / 1.28,
+// 1000 1.50 / 1.20; n = 3,200: 1.34 / 1.09, 1.31 / 1.06; n = 4,000: W = 50 1.35 / 1.22, 100 1.18 /
+// 0.94, 1000 1.04 / 0.82; n = 5,000: W = 10 1.39 / 1.24, 50 1.13 / 1.01, 100 0.93 / 0.76; n =
+// 6,007: W = 50 1.06 / 0.93, 100 0.82 / 0.69; n = 8,000: W = 10 0.88 / 0.77, 25 0.94 / 0.80; n =
+// 10,500: W = 1 0.68 / 0.62, 10 0.63 / 0.55; n = 12,000: W = 10 0.54 / 0.47; at n = 6,600, W = 10
+// 1.04 / 0.91, and 1.10 on WS k = 10.  So: at most 7,200 nodes whatever the lengths, and n min(W, 200)^0.35 <= 19,500, the crossover of the ER graphs
+// (n = 5,000 for W = 50, 3,900 for W = 100, 3,050 for W >= 200).  Per-edge length ranges and
+// length laws count as W = 65,535.
 bool steps_beat_buckets(const afc_mc_problem &p) {
   const double w = (p.w_hi || p.wtab_ptr) ? 65535.0 : (double)std::max<uint32_t>(p.w_hi_all, 1u);
-  return (double)p.n * std::pow(std::min(w, 200.0), 0.35) <= 19500.0;
+  return p.n <= 7200 && (double)p.n * std::pow(std::min(w, 200.0), 0.35) <= 19500.0;
 }
 
 // Launch plan of the global-memory path for one problem.

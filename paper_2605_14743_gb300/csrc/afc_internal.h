@@ -110,9 +110,6 @@ cudaError_t launch_certificates(const ChainDev &C, const double *mu0, const doub
                                 const int32_t *piv0, double eps_bar, double r_min, int32_t npairs,
                                 const int32_t *pu, const int32_t *pv, double *gap, double *sharp,
                                 unsigned char *ws, const SolveWs &L, cudaStream_t stream);
-// The right-hand side y0 = s_C + s_U Q_UC of the reduced solve (part: 64 c doubles of scratch).
-void launch_nominal_rhs(const ChainDev &C, const double *rowscale, double *part, double *y,
-                        cudaStream_t stream);
 // Device memory of one sweep CTA, and of the nominal matrix's FP32 inverse and its transpose.
 size_t perturb_slab_bytes(int32_t n, int32_t c);
 size_t perturb_inverse_bytes(int32_t c);

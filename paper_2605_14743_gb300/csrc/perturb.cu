@@ -17,7 +17,7 @@
 // costs one FP64 multiply-add.  The rows' (N' 1)_i are screened in FP32; the ones that can be the
 // maximum are computed in FP64.  Measured, before (8 FP64 operations per entry, a factorisation or
 // two chains of triangular solves per round, (N' 1) by a thread per row) and now: c = 97, n = 1,000,
-// 2,000 perturbations 13.4 -> 4.9 ms; c = 751, n = 3,000, 304 perturbations 30.8 -> 8.9 ms, its
+// 2,000 perturbations 13.4 -> 4.8 ms; c = 751, n = 3,000, 304 perturbations 30.8 -> 8.2 ms, its
 // kernel with the FP64 pipe 47% and issue 31% active (16 warps per SM wait for loads and chains).
 #include <algorithm>
 #include <cstdint>
@@ -213,7 +213,7 @@ __device__ __forceinline__ int32_t draw(uint32_t j, uint32_t i, uint32_t p, uint
 // product instead of two chains of 2 c / 32 dependent blocks.  Once per launch.
 constexpr int kInvThreads = 256;
 __host__ __device__ inline size_t inverse_smem(int32_t c, int nr) {
-  return sizeof(float) * ((((size_t)c * nr + 31) & ~size_t(31)) + 256 * 33 + 32 * 33);
+  return sizeof(float) * ((((size_t)c * nr + 31) & ~size_t(31)) + 256 * 33 + 2 * 32 * 33);
 }
 
 template <int NR>
@@ -222,10 +222,12 @@ inverse32_kernel(const double *lu, const int32_t *piv, int32_t c, size_t ld, flo
   extern __shared__ __align__(16) float fsm[];
   float *X = fsm;                                                     // [c][NR]
   float *tile = X + (((size_t)c * NR + 31) & ~size_t(31));            // [256][33]
-  float *D = tile + 256 * 33;                                         // [32][33]
+  float *diag = tile + 256 * 33;                                      // [2][32][33]
+  __shared__ int32_t first;
   const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int32_t j0 = (int32_t)blockIdx.x * NR;
   for (int32_t q = tid; q < c * NR; q += kInvThreads) X[q] = 0.0f;
+  if (tid == 0) first = c;
   __syncthreads();
   if (tid < NR && j0 + tid < c) {   // the unit vector through the row swaps
     int32_t pos = j0 + tid;
@@ -235,7 +237,18 @@ inverse32_kernel(const double *lu, const int32_t *piv, int32_t c, size_t ld, flo
       else if (pos == q) pos = k;
     }
     X[pos * NR + tid] = 1.0f;
+    atomicMin(&first, pos);
   }
+  __syncthreads();
+  // diagonal block kb into one of two buffers: the next block's is loaded during the update
+  auto stage = [&](int32_t kb, bool lower, float *D) {
+    const int nb = min(32, c - kb);
+    for (int q = tid; q < 32 * 32; q += kInvThreads) {
+      const int i = q >> 5, j = q & 31;
+      D[i * 33 + j] = i < nb && j < nb && (lower ? j < i : j >= i)
+                          ? trunc_f32(lu[(size_t)(kb + i) * c + kb + j]) : 0.0f;
+    }
+  };
   // rows [r0, r0 + 256) take their products with the block's NR columns off; a warp stages the
   // rows that its own lanes use
   auto update = [&](int32_t first, int32_t last, int32_t kb, int nb) {
@@ -263,12 +276,12 @@ inverse32_kernel(const double *lu, const int32_t *piv, int32_t c, size_t ld, flo
       __syncwarp();
     }
   };
-  for (int32_t kb = 0; kb < c; kb += 32) {                            // L, unit lower
+  int buf = 0;
+  const int32_t kb0 = first / 32 * 32;   // the columns are zero above
+  stage(kb0, true, diag);
+  for (int32_t kb = kb0; kb < c; kb += 32) {                          // L, unit lower
     const int nb = min(32, c - kb);
-    for (int q = tid; q < 32 * 32; q += kInvThreads) {
-      const int i = q >> 5, j = q & 31;
-      D[i * 33 + j] = i < nb && j < i ? trunc_f32(lu[(size_t)(kb + i) * c + kb + j]) : 0.0f;
-    }
+    const float *D = diag + buf * 32 * 33;
     __syncthreads();
     if (warp < NR) {
       float v = lane < nb ? X[(kb + lane) * NR + warp] : 0.0f;
@@ -276,14 +289,14 @@ inverse32_kernel(const double *lu, const int32_t *piv, int32_t c, size_t ld, flo
       if (lane < nb) X[(kb + lane) * NR + warp] = v;
     }
     __syncthreads();
+    buf ^= 1;
+    if (kb + 32 < c) stage(kb + 32, true, diag + buf * 32 * 33);
+    else stage(kb, false, diag + buf * 32 * 33);   // the last block again, for U
     update(kb + nb, c, kb, nb);
   }
   for (int32_t kb = ((c - 1) / 32) * 32; kb >= 0; kb -= 32) {         // U
     const int nb = min(32, c - kb);
-    for (int q = tid; q < 32 * 32; q += kInvThreads) {
-      const int i = q >> 5, j = q & 31;
-      D[i * 33 + j] = i < nb && j >= i && j < nb ? trunc_f32(lu[(size_t)(kb + i) * c + kb + j]) : 0.0f;
-    }
+    const float *D = diag + buf * 32 * 33;
     __syncthreads();
     if (warp < NR) {
       const float d = lane < nb ? 1.0f / D[lane * 33 + lane] : 0.0f;
@@ -295,6 +308,8 @@ inverse32_kernel(const double *lu, const int32_t *piv, int32_t c, size_t ld, flo
       if (lane < nb) X[(kb + lane) * NR + warp] = v * d;
     }
     __syncthreads();
+    buf ^= 1;
+    if (kb > 0) stage(kb - 32, false, diag + buf * 32 * 33);
     update(0, kb, kb, nb);
   }
   __syncthreads();
@@ -361,70 +376,71 @@ __device__ __forceinline__ Pair pair_fma(Pair a, double x, double y) {
   a.l += fma(x, y, -p);
   return a;
 }
-constexpr int kDefectChunks = 32;
+constexpr int kDefectChunks = 128;
 
-// part [chunks][2][c]: sums over the rows outside C and over those of C (a thread per column).
-__global__ void __launch_bounds__(128)
-nominal_defect_kernel(ChainDev C, const double *rowscale, const double *mu0, Pair *part) {
+// part [chunks][2][c]: column sums of a chunk of rows, those outside C and those of C.  One CTA per
+// chunk, a row at a time (its columns are distinct), from the sparse rows the solve left.
+__global__ void __launch_bounds__(256)
+nominal_defect_kernel(ChainDev C, const int32_t *nzptr, const int32_t *nzcol, const double *nzval,
+                      const double *mu0, Pair *part) {
   const int32_t n = C.n, c = C.c;
-  const int32_t pj = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x);
-  if (pj >= c) return;
-  const size_t stride = (size_t)n + 1;
-  const int32_t per = (n + (int32_t)gridDim.y - 1) / (int32_t)gridDim.y;
-  const int32_t i0 = (int32_t)blockIdx.y * per, i1 = min(n, i0 + per);
-  const uint32_t *col = C.counts + C.c_list[pj];
+  const int32_t per = (n + (int32_t)gridDim.x - 1) / (int32_t)gridDim.x;
+  const int32_t i0 = (int32_t)blockIdx.x * per, i1 = min(n, i0 + per);
+  Pair *u = part + (size_t)blockIdx.x * 2 * c, *a = u + c;
   const double unif = 1.0 / (double)n;
-  Pair u{0.0, 0.0}, a{0.0, 0.0};
-  for (int32_t i = i0; i < i1; i += 8) {
-    uint32_t v[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) v[k] = i + k < i1 ? col[(size_t)(i + k) * stride] : 0u;
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (v[k]) {
-        const double q = rowscale[2 * (i + k)] * (double)v[k];
-        if (C.c_index[i + k] >= 0) a = pair_fma(a, mu0[i + k], q);
-        else u = pair_fma(u, C.s ? C.s[i + k] : unif, q);
-      }
+  for (int32_t k = (int32_t)threadIdx.x; k < 2 * c; k += (int32_t)blockDim.x) u[k] = Pair{0.0, 0.0};
+  __syncthreads();
+  for (int32_t i = i0; i < i1; ++i) {
+    const int32_t e0 = nzptr[i], len = nzptr[i + 1] - 1 - e0;
+    const bool in_c = C.c_index[i] >= 0;
+    const double w = in_c ? mu0[i] : C.s ? C.s[i] : unif;
+    Pair *to = in_c ? a : u;
+    for (int32_t k = (int32_t)threadIdx.x; k < len; k += (int32_t)blockDim.x) {
+      const int32_t pj = nzcol[e0 + k];
+      to[pj] = pair_fma(to[pj], w, nzval[e0 + k]);
+    }
+    __syncthreads();
   }
-  part[((size_t)blockIdx.y * 2) * c + pj] = u;
-  part[((size_t)blockIdx.y * 2 + 1) * c + pj] = a;
 }
 
-// Sums the parts (warp lanes stride the columns) and, a warp per row, rho_t.
+__device__ __forceinline__ Pair warp_pair_sum(Pair r) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double h = __shfl_xor_sync(0xFFFFFFFFu, r.h, o), l = __shfl_xor_sync(0xFFFFFFFFu, r.l, o);
+    r = pair_add(r, h);
+    r.l += l;
+  }
+  return r;
+}
+
+// A warp per observed state: its column's parts, and its row's defect rho_t.
 __global__ void __launch_bounds__(256)
 nominal_finish_kernel(ChainDev C, const double *mu0, const Pair *part, int chunks,
                       const int32_t *nzptr, const int32_t *nzcol, const double *nzval,
                       const double *t0, double *y0, double *rho, double *rho_t) {
-  const int32_t c = C.c, at = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x);
-  const int32_t step = (int32_t)(gridDim.x * blockDim.x);
-  for (int32_t pj = at; pj < c; pj += step) {
-    Pair u{C.s ? C.s[C.c_list[pj]] : 1.0 / (double)C.n, 0.0};
-    Pair a{0.0, 0.0};
-    for (int k = 0; k < chunks; ++k) {
-      const Pair pu = part[((size_t)k * 2) * c + pj], pa = part[((size_t)k * 2 + 1) * c + pj];
+  const int32_t c = C.c, lane = (int32_t)(threadIdx.x & 31u);
+  const int32_t step = (int32_t)((gridDim.x * blockDim.x) >> 5);
+  for (int32_t b = (int32_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); b < c; b += step) {
+    const int32_t i = C.c_list[b], e0 = nzptr[i], len = nzptr[i + 1] - 1 - e0;
+    Pair u{0.0, 0.0}, a{0.0, 0.0}, r{0.0, 0.0};
+    for (int k = lane; k < chunks; k += 32) {
+      const Pair pu = part[(size_t)k * 2 * c + b], pa = part[((size_t)k * 2 + 1) * c + b];
       u = pair_add(u, pu.h);
       u.l += pu.l;
       a = pair_add(a, pa.h);
       a.l += pa.l;
     }
-    y0[pj] = u.h + u.l;
-    u = pair_add(pair_add(u, a.h), -mu0[C.c_list[pj]]);
-    rho[pj] = u.h + (u.l + a.l);
-  }
-  const int32_t lane = at & 31;
-  for (int32_t b = at >> 5; b < c; b += step >> 5) {
-    const int32_t i = C.c_list[b], e0 = nzptr[i], len = nzptr[i + 1] - 1 - e0;
-    Pair r{0.0, 0.0};
     for (int32_t k = lane; k < len; k += 32) r = pair_fma(r, nzval[e0 + k], t0[nzcol[e0 + k]]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double h = __shfl_xor_sync(0xFFFFFFFFu, r.h, o), l = __shfl_xor_sync(0xFFFFFFFFu, r.l, o);
-      r = pair_add(r, h);
-      r.l += l;
+    u = warp_pair_sum(u);
+    a = warp_pair_sum(a);
+    r = pair_add(pair_add(warp_pair_sum(r), 1.0), -t0[b]);
+    if (lane == 0) {
+      u = pair_add(u, C.s ? C.s[i] : 1.0 / (double)C.n);
+      y0[b] = u.h + u.l;
+      u = pair_add(pair_add(u, a.h), -mu0[i]);
+      rho[b] = u.h + (u.l + a.l);
+      rho_t[b] = r.h + r.l;
     }
-    r = pair_add(pair_add(r, 1.0), -t0[b]);
-    if (lane == 0) rho_t[b] = r.h + r.l;
   }
 }
 
@@ -1300,10 +1316,10 @@ cudaError_t launch_perturb(const ChainDev &C, const afc_perturb_params &pp, cons
                                                         rank0, byrank0);
   double *rho = reinterpret_cast<double *>(ws + L.off_tmp + 512), *rho_t = rho + c;   // 4 n + 4 c there
   if (c > 0) {
-    const int chunks = std::min(n, kDefectChunks);
+    const int chunks = (int)std::max<size_t>(
+        1, std::min({(size_t)n, (size_t)kDefectChunks, (L.total - L.off_slab) / (2 * sizeof(Pair) * (size_t)c)}));
     Pair *part = reinterpret_cast<Pair *>(ws + L.off_slab);
-    nominal_defect_kernel<<<dim3((unsigned)((c + 127) / 128), (unsigned)chunks), 128, 0, stream>>>(
-        C, reinterpret_cast<const double *>(ws + L.off_rowscale), mu0, part);
+    nominal_defect_kernel<<<chunks, 256, 0, stream>>>(C, nzptr, nzcol, nzval, mu0, part);
     nominal_finish_kernel<<<std::min((c + 7) / 8, 608), 256, 0, stream>>>(C, mu0, part, chunks, nzptr,
                                                                          nzcol, nzval, t0, y0, rho, rho_t);
   }

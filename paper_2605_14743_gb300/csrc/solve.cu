@@ -317,15 +317,6 @@ chain_rows_kernel(ChainDev C, const double *t, const int32_t *nzptr, const int32
   if (lane == 0 && best) atomicMax(reinterpret_cast<unsigned long long *>(&scalars[2]), best);
 }
 
-void launch_nominal_rhs(const ChainDev &C, const double *rowscale, double *part, double *y,
-                        cudaStream_t stream) {
-  if (C.c <= 0) return;
-  const int chunks = std::min(C.n, 64);
-  const unsigned blocks = (unsigned)((C.c + 127) / 128);
-  u_rows_kernel<<<dim3(blocks, (unsigned)chunks), 128, 0, stream>>>(C, rowscale, part);
-  y_kernel<<<blocks, 128, 0, stream>>>(C, part, chunks, y);
-}
-
 cudaError_t launch_solve(const ChainDev &C, double *mu, double *b, double *scalars, double *lu,
                          int32_t *piv, unsigned char *ws, const SolveWs &L, uint32_t *status_dev,
                          int smem_optin, cudaStream_t stream) {
@@ -344,7 +335,9 @@ cudaError_t launch_solve(const ChainDev &C, double *mu, double *b, double *scala
   exclusive_scan_kernel<<<1, 1024, 0, stream>>>(n, nnz_row, nzptr);
   row_fill_kernel<<<blocks, 256, 0, stream>>>(C, rowscale, nzptr, nzcol, nzval, lu, t);
   if (c > 0) {
-    launch_nominal_rhs(C, rowscale, part, y, stream);
+    const int chunks = std::min(n, 64);
+    u_rows_kernel<<<dim3((unsigned)((c + 127) / 128), (unsigned)chunks), 128, 0, stream>>>(C, rowscale, part);
+    y_kernel<<<(c + 127) / 128, 128, 0, stream>>>(C, part, chunks, y);
     const LuBatch B{lu, 0, piv, 0, y, t, nullptr, status_dev};
     cudaError_t e = launch_lu(B, c, 1, smem_optin, stream);
     if (e != cudaSuccess) return e;

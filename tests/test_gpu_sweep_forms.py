@@ -68,16 +68,19 @@ def test_sweep_forms(n, c, lengths, radius, r_min, flat, model, s):
 @pytest.mark.parametrize("n", [1, 31, 257])
 def test_rank_screen_keeps_the_band(n):
     """The FP32 screen of the ranking decides nothing inside the tie band: values equal, apart by
-    less than the band, by a little more, tiny, zero and beyond FP32's range."""
+    less than the band, by a little more, tiny, zero, beyond FP32's range and negative."""
     afc = pytest.importorskip("paper_2605_14743_gb300")
     rng = np.random.default_rng(n)
-    for top in (1.0, 1e200):
-        b = rng.choice([0.25, 0.25 + 1e-10, 0.25 + 1e-6, 0.5, 1e-45, 0.0, top], n)
+    for top, sign in ((1.0, 1.0), (1e200, 1.0), (1.0, -1.0)):
+        b = sign * rng.choice([0.25, 0.25 + 1e-10, 0.25 + 1e-6, 0.5, 1e-45, 0.0, top], n)
+        if sign < 0.0:
+            b -= 0.125
         tie = 1e-9
-        tau = tie * b.max()
+        tau = tie * max(b.max(), 0.0)   # the band's scale is at least 0
         d = b[:, None] - b[None, :]
         u = np.arange(n)
         before = (d > tau) | ((np.abs(d) <= tau) & (u[:, None] < u[None, :]))
+        np.fill_diagonal(before, False)
         ref = before.sum(axis=0)
         rank = torch.empty(n, dtype=torch.int32, device="cuda")
         topk = torch.empty(1, dtype=torch.int32, device="cuda")
@@ -85,3 +88,13 @@ def test_rank_screen_keeps_the_band(n):
                      torch.cuda.current_stream().cuda_stream)
         torch.cuda.synchronize()
         assert (rank.cpu().numpy() == ref).all()
+
+
+def test_sweep_uses_the_solved_chain():
+    """The sweep perturbs the chain that was solved, whatever has become of the counts since."""
+    counts = _counts(60, 33, [1, 31, 32, 33], 6000, 5, False)
+    ch = Chain(counts, 6000, 0.15)
+    a = ch.sweep(0, 4, 0.05, 0.05, 19)
+    ch.counts.zero_()
+    b = ch.sweep(0, 4, 0.05, 0.05, 19)
+    assert all((x == y).all() for x, y in zip(a, b))

@@ -328,7 +328,7 @@ cudaError_t launch_solve(const ChainDev &C, double *mu, double *b, double *scala
   int32_t *nzcol = reinterpret_cast<int32_t *>(ws + L.off_nzcol);
   double *nzval = reinterpret_cast<double *>(ws + L.off_nzval);
   int32_t *nnz_row = reinterpret_cast<int32_t *>(ws + L.off_flags);
-  double *part = reinterpret_cast<double *>(ws + L.off_slab);   // a slab holds n (c + 1) doubles
+  double *part = reinterpret_cast<double *>(ws + L.off_slab);   // the slabs hold 64 (c + 1) doubles
   const int64_t want_blocks = ((int64_t)n * 32 + 255) / 256;
   const int blocks = (int)(want_blocks < 2048 ? want_blocks : 2048);
   row_prep_kernel<<<blocks, 256, 0, stream>>>(C, rowscale, nnz_row);

@@ -576,8 +576,11 @@ __device__ __forceinline__ double move_row(const RowArgs &R, int32_t i, int32_t 
   dab = warp_sum_ll(dab);
   const double rec = dab > 0 ? recip(trunc_double(dab)) : 0.0;
   const float coef_f = R.radius_f * trunc_f32(rec);
-  // v = q + d coef in FP32, off by at most 5e-7 of the shift and 2e-7 of q; neg_bits: the entries
-  // that clip (those of the first 32 per lane)
+  // v = q + d coef in FP32, off by at most 5e-7 of the shift and 2e-7 of q.  An entry that clips has
+  // a shift of at least q, so 1e-5 q covers it; an absorption in [0, r_min) has a shift of at most
+  // q + r_min, so the floor's margin is 1e-6 q on top of 1e-4 r_min (a margin in r_min alone misses
+  // rows whose q is more than 240 r_min).  neg_bits: the entries that clip (those of the first 32
+  // per lane)
   bool general = R.always_general, close = R.always_general || nt > 32;
   uint32_t neg_bits = 0;
 #pragma unroll (kUnroll)
@@ -586,7 +589,7 @@ __device__ __forceinline__ double move_row(const RowArgs &R, int32_t i, int32_t 
     const float q0 = trunc_f32(val_of(s));
     const float v = fmaf(trunc_f32(d_of(s)), coef_f, q0), band = 4e-6f * q0;
     if (k < supp) {
-      general |= v < (k < supp - 1 ? 1e-5f * q0 : fmaxf(1e-5f * q0, R.floor_f));
+      general |= v < (k < supp - 1 ? 1e-5f * q0 : fmaxf(1e-5f * q0, fmaf(1e-6f, q0, R.floor_f)));
       if (v < -band) neg_bits |= 1u << (s & 31);
       close |= !(fabsf(v) > band);
     }

@@ -453,6 +453,7 @@ struct RowArgs {
   int32_t model;
   double radius, r_min, rel;
   float radius_f, floor_f;       // of the FP32 tests (floor_f: r_min and a margin)
+  float screen;                  // margin of the (N' 1) screen, in units of the largest t
   bool always_general;           // the radius is beyond what they cover
 };
 
@@ -1012,9 +1013,10 @@ perturb_kernel(ChainDev C, afc_perturb_params pp, const double *mu0, const doubl
   const double t0_max = block_max(pmx, red);
   double loc_db = 0.0, loc_lin = 0.0, loc_t = 0.0;
   RowArgs R{nzcol, C.c_list, nzval, c, (uint32_t)n, 0u, (uint32_t)pp.seed, (uint32_t)(pp.seed >> 32),
-            pp.model, pp.l1_radius, pp.r_min, pp.rel_radius, 0.0f, 0.0f, !(pp.l1_radius <= 1e6)};
+            pp.model, pp.l1_radius, pp.r_min, pp.rel_radius, 0.0f, 0.0f, 0.0f, !(pp.l1_radius <= 1e6)};
   R.radius_f = R.always_general ? 0.0f : trunc_f32(pp.l1_radius);
   R.floor_f = trunc_f32(pp.r_min) * 1.0001f;
+  R.screen = R.always_general ? 4e-7f : 1.2e-6f * fminf(R.radius_f, 2.0f) + 4e-7f;
   // the multiplicative moves of the robust search (50% an entry) rarely contract 5x a round; on chip
   // the factorisation is the cheaper try for them
   const bool try_defect = inv != nullptr && !(on_chip && pp.model == 1);
@@ -1124,6 +1126,7 @@ perturb_kernel(ChainDev C, afc_perturb_params pp, const double *mu0, const doubl
     }
     // (3) E'[T], max b', z . 1
     double pT = 0.0, pY = 0.0, pm = 0.0;
+    float tm = 0.0f;   // the largest (N' 1)_i on C, truncated
     for (int32_t v = threadIdx.x; v < n; v += blockDim.x) {
       const int32_t pv = C.c_index[v];
       pT += pv >= 0 ? X.mu[pv] : (C.s ? C.s[v] : s_unif);
@@ -1131,6 +1134,7 @@ perturb_kernel(ChainDev C, afc_perturb_params pp, const double *mu0, const doubl
     for (int32_t k = threadIdx.x; k < c; k += blockDim.x) {
       pY += z[k];
       X.rt[k] = trunc_f32(X.t[k]);
+      tm = fmaxf(tm, X.rt[k]);
       loc_t = fmax(loc_t, X.t[k]);
     }
     const double T = block_sum(pT, red);
@@ -1159,9 +1163,12 @@ perturb_kernel(ChainDev C, afc_perturb_params pp, const double *mu0, const doubl
     }
     const double bmax = block_max(pm, red);
     const double tau = pp.tie_rel * bmax;
-    // (4) the largest (N' 1)_i outside C: sum_j q'_ij t_j of every row in FP32 (all terms positive,
-    // so it is off by a few 1e-6 and by 2^-24 per addition), then in FP64 the rows within twice
-    // that of the largest
+    // (4) the largest (N' 1)_i outside C: S_i = sum_j q'_ij t_j of every row in FP32, then in FP64 the
+    // rows that can hold the maximum over all rows.  With t at most tm, the FP32 S_i is off by
+    //   tm (5e-7 sum_j |shift_j| + 2e-7) for the entries (move_row's bounds; the shifts of the entries
+    // kept sum to at most 2 after the row's scaling, whatever the radius) and, all terms being
+    // positive, by S_i (4e-7 + 2^-24 (c / 32 + 7)) for t, the scaling and the additions, S_i <= tm.
+    // Two rows' errors count, and a row below tm - 1 is below the rows of C.
     float best = 0.0f;
     for (int32_t i0 = warp; i0 < n; i0 += 4 * nw) {
       float part[4];
@@ -1199,10 +1206,14 @@ perturb_kernel(ChainDev C, afc_perturb_params pp, const double *mu0, const doubl
     }
 #pragma unroll
     for (int o = 16; o > 4; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xFFFFFFFFu, best, o));
-    if (lane == 0) fred[warp] = best;
+    tm = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(tm)));   // not negative
+    if (lane == 0) { fred[2 * warp] = best; fred[2 * warp + 1] = tm; }
     __syncthreads();
-    for (int32_t w = 0; w < nw; ++w) best = fmaxf(best, fred[w]);
-    const float least = best * (1.0f - (6e-6f + 2.5e-7f * (float)(c / 32 + 1)));
+    for (int32_t w = 0; w < nw; ++w) {
+      best = fmaxf(best, fred[2 * w]);
+      tm = fmaxf(tm, fred[2 * w + 1]);
+    }
+    const float least = fmaxf(best, tm - 1.0f) - tm * (2e-6f + R.screen + 2.5e-7f * (float)(c / 32 + 1));
     for (int32_t i = warp; i < n; i += nw) {
       if (C.c_index[i] >= 0 || !(sf[i] >= least)) continue;
       const int32_t e0 = nzptr[i];

@@ -1,5 +1,5 @@
 """The FP32 screens of the perturbation sweep decide nothing that FP64 decides otherwise: rows whose
-absorption ends just below the floor."""
+absorption ends just below the floor, rows that lose nearly all of their transient mass."""
 import numpy as np
 import pytest
 
@@ -63,3 +63,25 @@ def test_rows_just_below_the_absorption_floor(c, r_min, radius):
     bo, mx, ref = _sweep(counts, p, radius, r_min)
     assert close(bo, ref.b)
     assert max_rel(mx, [ref.max_db, ref.max_lin_err, ref.max_rowsum_N]) < 1e-9
+
+
+def test_longest_walk_among_rows_that_cancel():
+    """Every row has one transient entry that loses 0.4 of its 0.401, so the FP32 sums of the rows
+    outside C are off by 1e-4 of themselves; one of them is larger by 3e-8 and holds the maximum."""
+    n, radius, r_min = 7, 0.8, 0.05
+    found = 0
+    for p in range(4000):
+        sh = [_shifts(i, p, [0, n], radius)[0] for i in range(n)]
+        if max(sh) > 0.0:
+            continue   # both shifts of a row are +-0.4
+        for top in (1, 4):
+            counts = np.zeros((n, n + 1), np.uint32)
+            for i in range(n):
+                counts[i] = _row(n, [0], 1.0 - (0.001 if i == 0 else 0.401 + 3e-8 * (i == top)))
+            bo, mx, ref = _sweep(counts, p, radius, r_min)
+            assert close(bo, ref.b)
+            assert max_rel(mx, [ref.max_db, ref.max_lin_err, ref.max_rowsum_N]) < 1e-9
+        found += 1
+        if found == 6:
+            return
+    assert False, "no perturbation moves every row down"

@@ -248,6 +248,7 @@ mc_counts_kernel(const McDev *__restrict__ probs, int nprob, uint64_t *item_pref
       }
       __syncthreads();
       if (ctl->wide_redo) {
+        __syncthreads();   // every thread has read the flag before the next attempt clears it
         wide = true;
         if (threadIdx.x == 0 && P.stats) atomicAdd(u64p(&P.stats->wide_redone), 1ull);
         continue;

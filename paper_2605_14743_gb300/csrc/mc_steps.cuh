@@ -247,14 +247,23 @@ __device__ __forceinline__ void level_order(const StepSlot &sl, uint32_t n, uint
     base += total;
   }
   __syncwarp();
-  for (uint32_t v = lane; v < n; v += 32) {
-    const uint32_t w = sl.dist[v];
-    if (w & kFlag) {
-      const uint32_t pos = atomicAdd(at((w & kMask) >> dbits), 1u) & 0xFFFFu;
-      *ord_at<COMPACT>(sl, pos) = (uint16_t)v;
+  // A compact slot's counter is one half of a word whose other half takes an order entry: all
+  // counters of a group of nodes first, then the entries, the warp together in between.
+  constexpr int kGroup = 4;
+  for (uint32_t v0 = 0; v0 < n; v0 += 32u * kGroup) {
+    uint32_t pos[kGroup];
+#pragma unroll
+    for (int t = 0; t < kGroup; ++t) {
+      const uint32_t v = v0 + 32u * t + lane;
+      const uint32_t w = v < n ? sl.dist[v] : 0u;
+      pos[t] = w & kFlag ? atomicAdd(at((w & kMask) >> dbits), 1u) & 0xFFFFu : n;
     }
+    __syncwarp();
+#pragma unroll
+    for (int t = 0; t < kGroup; ++t)
+      if (pos[t] < n) *ord_at<COMPACT>(sl, pos[t]) = (uint16_t)(v0 + 32u * t + lane);
+    __syncwarp();
   }
-  __syncwarp();
   // a level's counter now holds its end, i.e. the start of the next one (no level is empty)
   for (uint32_t l = lane; l <= lmax; l += 32) {
     const uint32_t start = l ? level_get<COMPACT>(at(l - 1u)) : 0u;

@@ -864,15 +864,18 @@ __device__ inline void realize_csr(const McDev &P, uint32_t r, uint32_t *rp, uin
 
 // realize_csr for a realization built on chip: each arc is drawn once (an arc per thread, or a
 // node's arcs per thread in the hop mode) into tmp [2 m] (shared memory), then compacted.  Small
-// graphs spend most of their time in such per-realization phases.
+// graphs spend most of their time in such per-realization phases.  An arc of a row with a bad edge
+// or neighbour is an error wherever it lies, as in realize_csr, and arcs outside all rows are not read.
 __device__ inline void realize_csr_chip(const McDev &P, uint32_t r, uint32_t *rp, uint32_t *arc,
                                         uint32_t *tmp, CtaHead *ctl, const uint32_t *hop) {
   constexpr uint32_t kDead = 0xFFFFFFFFu;   // no alive arc: length 65535 to node 65535 >= n
   const uint32_t n = P.n, arcs = (uint32_t)(2 * P.m), T = blockDim.x;
+  const int32_t first = max(P.row_ptr[0], 0), last = min(P.row_ptr[n], (int32_t)arcs);
   uint32_t wmax = 1, err = 0;
-  auto draw = [&](uint32_t a) -> uint32_t {
+  auto draw = [&](int32_t a, bool near) -> uint32_t {   // near: v's row is within the hop radius
     const uint32_t e = (uint32_t)P.eid[a], u = (uint32_t)P.col[a];
     if (e >= (uint64_t)P.m || u >= n) { err = kErrInput; return kDead; }
+    if (!near || (hop && hop[u] > P.hop_radius)) return kDead;
     bool alive; uint32_t w;
     edge_draw(P, r, e, alive, w);
     if (!alive) return kDead;
@@ -880,23 +883,25 @@ __device__ inline void realize_csr_chip(const McDev &P, uint32_t r, uint32_t *rp
     wmax = max(wmax, w);
     return u | (w << 16);
   };
+  // v's arcs; a row that leaves [first, last) is cut there, an error
+  auto row = [&](uint32_t v, auto &&f) {
+    const int32_t b0 = P.row_ptr[v], b1 = P.row_ptr[v + 1];
+    if (b0 < b1 && (b0 < first || b1 > last)) err = kErrInput;
+    for (int32_t a = max(b0, first); a < min(b1, last); ++a) f(a);
+  };
   if (hop) {
-    for (uint32_t v = threadIdx.x; v < n; v += T)
-      for (int32_t a = P.row_ptr[v]; a < P.row_ptr[v + 1]; ++a) {
-        if (a < 0 || (uint32_t)a >= arcs) { err = kErrInput; continue; }
-        const uint32_t u = (uint32_t)P.col[a];
-        tmp[a] = hop[v] > P.hop_radius || u >= n || hop[u] > P.hop_radius ? kDead : draw((uint32_t)a);
-      }
+    for (uint32_t v = threadIdx.x; v < n; v += T) {
+      const bool near = hop[v] <= P.hop_radius;
+      row(v, [&](int32_t a) { tmp[a] = draw(a, near); });
+    }
   } else {
-    for (uint32_t a = threadIdx.x; a < arcs; a += T) tmp[a] = draw(a);
+    for (int32_t a = first + (int32_t)threadIdx.x; a < last; a += (int32_t)T) tmp[a] = draw(a, true);
   }
   __syncthreads();
   const uint32_t per = (n + T - 1) / T;
   const uint32_t v0 = min(n, threadIdx.x * per), v1 = min(n, v0 + per);
   auto each = [&](uint32_t v, auto &&f) {
-    const int32_t a0 = max(P.row_ptr[v], 0), a1 = min(P.row_ptr[v + 1], (int32_t)arcs);
-    for (int32_t a = a0; a < a1; ++a)
-      if (tmp[a] != kDead) f(tmp[a]);
+    row(v, [&](int32_t a) { if (tmp[a] != kDead) f(tmp[a]); });
   };
   uint32_t cnt = 0;
   for (uint32_t v = v0; v < v1; ++v) each(v, [&](uint32_t) { ++cnt; });

@@ -338,7 +338,8 @@ int afc_bootstrap(const afc_chain *chain, const int32_t *next_states, const int3
  * the row's observed support (q_ij = 0 elsewhere); 0: on every j (new transitions up to eps).
  * Solved exactly per row (lower bounds, then the budget to the most negative coefficients
  * v_j - v_bot first, ties by j).  DEVICE in: counts [n][n+1], v [n].  DEVICE out: T [n],
- * Qstar [n][n] a minimising kernel (or NULL).  Workspace: 256 bytes.  SYNCHRONISES `stream`.
+ * Qstar [n][n] a minimising kernel (or NULL).  Workspace: 256 bytes (T holds the columns' order
+ * while the rows are solved: T and v do not overlap).  SYNCHRONISES `stream`.
  * Errors: AFC_EINVAL when some U_i is empty (its lower bounds exceed 1 - r_min). */
 int afc_robust_inner(const afc_chain *chain, const uint32_t *counts, double eps, double r_min,
                      int32_t support_only, const double *v, double v_bot, double *T, double *Qstar,

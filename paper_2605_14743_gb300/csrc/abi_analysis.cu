@@ -197,20 +197,15 @@ int afc_robust_inner(const afc_chain *chain, const uint32_t *counts, double eps,
   if (!workspace || workspace_bytes < 256) return fail(AFC_ENOMEM, "need 256 bytes of workspace");
   cudaStream_t s = (cudaStream_t)stream;
   uint32_t *status = static_cast<uint32_t *>(workspace);
-  AFC_CUDA(cudaMemsetAsync(status, 0, sizeof(uint32_t), s));
-  int32_t *order = nullptr;   // the columns' common order: the caller's workspace has no room
-  if (cudaMallocAsync(&order, sizeof(int32_t) * (size_t)chain->n, s) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return fail(AFC_ENOMEM, "device allocation");
-  }
-  cudaError_t e = launch_robust_inner(chain->n, chain->realizations, chain->alpha,
-                                      chain->absorb_floor, counts, eps, r_min, support_only ? 1 : 0,
-                                      v, v_bot, 1.0, order, T, Qstar, status, s);
+  uint32_t *arrived = status + 32;
+  AFC_CUDA(cudaMemsetAsync(status, 0, 256, s));
+  AFC_CUDA(launch_robust_inner_in_place(chain->n, chain->realizations, chain->alpha,
+                                        chain->absorb_floor, counts, eps, r_min, support_only ? 1 : 0,
+                                        v, v_bot, T, Qstar, status, arrived, dev_info().sms, s));
   uint32_t h = 0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&h, status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
-  cudaFreeAsync(order, s);
-  if (e != cudaSuccess) return cuda_fail(e, "robust inner launch");
+  AFC_CUDA(cudaMemcpyAsync(&h, status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
   AFC_CUDA(cudaStreamSynchronize(s));
+  if (h & kErrPassLimit) return fail(AFC_EDEVICE, "robust inner: the grid did not meet at its barrier");
   if (h) return fail(AFC_EINVAL, "empty uncertainty set: a row's lower bounds exceed 1 - r_min");
   return AFC_OK;
 }

@@ -129,6 +129,12 @@ cudaError_t launch_robust_inner(int32_t n, uint32_t R, double alpha, double eta,
                                 int support_only, const double *v, double v_bot, double vsign,
                                 int32_t *order, double *T, double *Qstar, uint32_t *status,
                                 cudaStream_t stream);
+// The inner problem (vsign 1) whose column order stands in T meanwhile; arrived: 0, on the device.
+cudaError_t launch_robust_inner_in_place(int32_t n, uint32_t R, double alpha, double eta,
+                                         const uint32_t *counts, double eps, double r_min,
+                                         int support_only, const double *v, double v_bot, double *T,
+                                         double *Qstar, uint32_t *status, uint32_t *arrived,
+                                         int num_sms, cudaStream_t stream);
 cudaError_t launch_robust_eval(int32_t n, const double *Qstar, double *A, int32_t *piv,
                                const double *f, const double *s, double *V, double *x, double *mu,
                                double *diff, uint32_t *status, int smem_optin, cudaStream_t stream);

@@ -8,6 +8,8 @@
 //                        budget goes to the entries in ascending order of v_j - v_bot (ties by
 //                        j) while that coefficient is negative, each up to its upper bound.  The
 //                        order is the same for every row (robust_order_kernel).
+//                        robust_inner_in_place_kernel does both in one launch for callers without
+//                        room for the order
 //   launch_robust_eval   A = I - Q*, its LU over the whole GPU (dense_lu.cu) with f and s in the
 //                        elimination, V = A^-1 f and the change of V; the robust value comes from
 //                        policy iteration on the host (inner problem at V, evaluate, until V stops
@@ -89,76 +91,143 @@ __device__ __forceinline__ uint32_t count_negative(int32_t n, const double *v, d
   return __reduce_add_sync(0xFFFFFFFFu, k);
 }
 
-// Row-wise inner problem (warp per row, rows warp, warp + nwarps, ...) at the continuation
-// value vsign * (v, v_bot): the budget is handed out 32 columns of the common order at a time, by
-// a prefix sum of their caps.  (Searching the next column for each row cost n per column: 550 us
-// at n = 500.)
+// Row i of the inner problem by one warp at the continuation value vsign * (v, v_bot) (vb = vsign
+// v_bot, nneg = count_negative): the budget is handed out 32 columns of the common order at a time,
+// by a prefix sum of their caps.  (Searching the next column for each row cost n per column: 550 us
+// at n = 500.)  Every lane gets T_i.
+__device__ double inner_row(uint32_t i, int32_t n, uint32_t R, double alpha, double eta,
+                            const uint32_t *counts, double eps, double r_min, int support_only,
+                            const double *v, double vb, double vsign, const int32_t *order,
+                            uint32_t nneg, double *Qstar, uint32_t *status) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t *row = counts + (size_t)i * ((size_t)n + 1);
+  const double scale = row_scale_warp(row, n, R, alpha, eta);
+  double *qs = Qstar ? Qstar + (size_t)i * n : nullptr;
+  // every entry at its lower bound
+  double base = 0.0, low = 0.0;
+  for (int32_t j = lane; j < n; j += 32) {
+    const uint32_t k = row[j];
+    double l = 0.0;
+    if (k) {
+      const double q = scale * (double)k;
+      l = q > eps ? q - eps : 0.0;
+      base += l * (vsign * v[j] - vb);
+      low += l;
+    }
+    if (qs) qs[j] = l;
+  }
+  base = warp_sum_d(base);
+  low = warp_sum_d(low);
+  __syncwarp();   // the lower bounds written by every lane, before the budget is added
+  double budget = (1.0 - r_min) - low;
+  if (budget < -1e-12) {
+    if (lane == 0) atomicOr(status, kErrInput);   // U_i is empty
+    budget = 0.0;
+  }
+  // the budget to the most negative coefficients first, each entry up to its upper bound
+  double acc = 0.0;
+  for (uint32_t k0 = 0; k0 < nneg && budget > 0.0; k0 += 32) {
+    const uint32_t k = k0 + lane;
+    int32_t j = 0;
+    double cap = 0.0;
+    if (k < nneg) {
+      j = order[k];
+      const double q = scale * (double)row[j];
+      if (q > 0.0) cap = fmin(q + eps, 1.0) - (q > eps ? q - eps : 0.0);
+      else if (!support_only) cap = fmin(eps, 1.0);
+      if (!(cap > 0.0)) cap = 0.0;
+    }
+    if (!__any_sync(0xFFFFFFFFu, cap > 0.0)) continue;
+    double incl = cap;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+      if (lane >= (uint32_t)o) incl += y;
+    }
+    double before = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
+    if (lane == 0) before = 0.0;
+    const double d = fmin(cap, fmax(budget - before, 0.0));
+    if (d > 0.0) {
+      acc += d * (vsign * v[j] - vb);
+      if (qs) qs[j] += d;
+    }
+    budget -= __shfl_sync(0xFFFFFFFFu, incl, 31);
+  }
+  return vsign * (vb + base + warp_sum_d(acc));
+}
+
+// The rows warp, warp + nwarps, ...
 __device__ void inner_rows(int32_t n, uint32_t R, double alpha, double eta,
                            const uint32_t *counts, double eps, double r_min, int support_only,
                            const double *v, double v_bot, double vsign, const int32_t *order,
                            double *T, double *Qstar, uint32_t *status, uint32_t warp,
                            uint32_t nwarps) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const size_t stride = (size_t)n + 1;
+  if (warp >= (uint32_t)n) return;
   const double vb = vsign * v_bot;
-  uint32_t nneg = 0xFFFFFFFFu;
+  const uint32_t nneg = count_negative(n, v, vb, vsign);
   for (uint32_t i = warp; i < (uint32_t)n; i += nwarps) {
-    if (nneg == 0xFFFFFFFFu) nneg = count_negative(n, v, vb, vsign);
-    const uint32_t *row = counts + (size_t)i * stride;
-    const double scale = row_scale_warp(row, n, R, alpha, eta);
-    double *qs = Qstar ? Qstar + (size_t)i * n : nullptr;
-    // every entry at its lower bound
-    double base = 0.0, low = 0.0;
-    for (int32_t j = lane; j < n; j += 32) {
-      const uint32_t k = row[j];
-      double l = 0.0;
-      if (k) {
-        const double q = scale * (double)k;
-        l = q > eps ? q - eps : 0.0;
-        base += l * (vsign * v[j] - vb);
-        low += l;
-      }
-      if (qs) qs[j] = l;
+    const double t = inner_row(i, n, R, alpha, eta, counts, eps, r_min, support_only, v, vb, vsign,
+                               order, nneg, Qstar, status);
+    if ((threadIdx.x & 31u) == 0) T[i] = t;
+  }
+}
+
+// Waits until every CTA of a cooperative launch has come this far (arrived: 0 at the launch; want:
+// CTAs times the barriers so far).  False after about a second without them.
+__device__ bool grid_barrier(uint32_t *arrived, uint32_t want) {
+  __shared__ int met;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    atomicAdd(arrived, 1u);
+    int ok = 0;
+    for (uint32_t k = 0; k < (1u << 24) && !ok; ++k) {
+      ok = *reinterpret_cast<volatile uint32_t *>(arrived) >= want;
+      if (!ok) __nanosleep(64);
     }
-    base = warp_sum_d(base);
-    low = warp_sum_d(low);
-    __syncwarp();   // the lower bounds written by every lane, before the budget is added
-    double budget = (1.0 - r_min) - low;
-    if (budget < -1e-12) {
-      if (lane == 0) atomicOr(status, kErrInput);   // U_i is empty
-      budget = 0.0;
-    }
-    // the budget to the most negative coefficients first, each entry up to its upper bound
-    double acc = 0.0;
-    for (uint32_t k0 = 0; k0 < nneg && budget > 0.0; k0 += 32) {
-      const uint32_t k = k0 + lane;
-      int32_t j = 0;
-      double cap = 0.0;
-      if (k < nneg) {
-        j = order[k];
-        const double q = scale * (double)row[j];
-        if (q > 0.0) cap = fmin(q + eps, 1.0) - (q > eps ? q - eps : 0.0);
-        else if (!support_only) cap = fmin(eps, 1.0);
-        if (!(cap > 0.0)) cap = 0.0;
-      }
-      if (!__any_sync(0xFFFFFFFFu, cap > 0.0)) continue;
-      double incl = cap;
+    met = ok;
+    __threadfence();
+  }
+  __syncthreads();
+  return met != 0;
+}
+
+constexpr uint32_t kKeptRows = 64;   // rows per warp of the kernel below
+
+// The whole inner problem (vsign 1) without scratch of its own: the order of the columns, 4 n bytes,
+// stands in T until every row is done, and the rows' values wait in registers (lane k of a warp
+// keeps its rows k and k + 32).  One cooperative launch of at least n / (8 kKeptRows) CTAs of 8 warps.
+// A call takes 54 us at n = 500 and 279 at n = 3,000 (with the order in an allocation of the call's
+// own and two launches: 182 and 440).
+__global__ void __launch_bounds__(256)
+robust_inner_in_place_kernel(int32_t n, uint32_t R, double alpha, double eta, const uint32_t *counts,
+                             double eps, double r_min, int support_only, const double *v, double vb,
+                             double *T, double *Qstar, uint32_t *status, uint32_t *arrived) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+  int32_t *order = reinterpret_cast<int32_t *>(T);
+  order_columns(n, v, vb, 1.0, order, warp, nwarps);
+  bool ok = grid_barrier(arrived, gridDim.x);
+  double kept[2] = {0.0, 0.0};
+  if (ok && warp < (uint32_t)n) {
+    const uint32_t nneg = count_negative(n, v, vb, 1.0);
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const double y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= (uint32_t)o) incl += y;
+    for (int h = 0; h < 2; ++h)
+      for (uint32_t k = 0; k < 32; ++k) {
+        const uint32_t i = warp + (32u * h + k) * nwarps;
+        if (i >= (uint32_t)n) break;
+        const double t = inner_row(i, n, R, alpha, eta, counts, eps, r_min, support_only, v, vb, 1.0,
+                                   order, nneg, Qstar, status);
+        if (lane == k) kept[h] = t;
       }
-      double before = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
-      if (lane == 0) before = 0.0;
-      const double d = fmin(cap, fmax(budget - before, 0.0));
-      if (d > 0.0) {
-        acc += d * (vsign * v[j] - vb);
-        if (qs) qs[j] += d;
-      }
-      budget -= __shfl_sync(0xFFFFFFFFu, incl, 31);
-    }
-    acc = warp_sum_d(acc);
-    if (lane == 0) T[i] = vsign * (vb + base + acc);
+  }
+  ok = grid_barrier(arrived, 2 * gridDim.x) && ok;   // every row has read the order
+  if (!ok && threadIdx.x == 0) atomicOr(status, kErrPassLimit);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const uint32_t i = warp + (32u * h + lane) * nwarps;
+    if (ok && i < (uint32_t)n) T[i] = kept[h];
   }
 }
 
@@ -353,6 +422,24 @@ cudaError_t launch_robust_inner(int32_t n, uint32_t R, double alpha, double eta,
                                                 support_only, v, v_bot, vsign, order, T, Qstar,
                                                 status);
   return cudaGetLastError();
+}
+
+cudaError_t launch_robust_inner_in_place(int32_t n, uint32_t R, double alpha, double eta,
+                                         const uint32_t *counts, double eps, double r_min,
+                                         int support_only, const double *v, double v_bot, double *T,
+                                         double *Qstar, uint32_t *status, uint32_t *arrived,
+                                         int num_sms, cudaStream_t stream) {
+  int per_sm = 0;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, robust_inner_in_place_kernel, 256, 0);
+  if (e != cudaSuccess) return e;
+  const int64_t fit = (int64_t)std::max(1, per_sm) * std::max(1, num_sms);
+  const int64_t grid = std::min<int64_t>(((int64_t)n + 7) / 8, fit);
+  if ((int64_t)n > grid * 8 * kKeptRows) return cudaErrorInvalidConfiguration;   // counts beyond 280 GB
+  void *args[] = {&n, &R, &alpha, &eta, &counts, &eps, &r_min, &support_only, &v, &v_bot, &T, &Qstar,
+                  &status, &arrived};
+  e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(robust_inner_in_place_kernel),
+                                  dim3((unsigned)grid), dim3(256), args, 0, stream);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_robust_eval(int32_t n, const double *Qstar, double *A, int32_t *piv,

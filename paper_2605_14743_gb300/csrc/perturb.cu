@@ -46,10 +46,13 @@ size_t perturb_inverse_bytes(int32_t c) { return 2 * sizeof(float) * (size_t)(c 
 
 __host__ __device__ inline size_t up256(size_t x) { return (x + 255) & ~size_t(255); }
 
-// One CTA's device slab (byte offsets): the dense matrix and its FP32 copy of the factorisation
-// fallback, c-vectors, the perturbed C rows (FP64, c + 1 apart) and the other rows (FP32).
+// One CTA's device slab (byte offsets): c-vectors, the perturbed C rows (FP64, c + 1 apart), the
+// other rows (FP32) and the dense matrix of the factorisation fallback.  The fallback's FP32 copy
+// takes the C rows' place: they are in the matrix by then, and the next perturbation writes them
+// anew.  (With a place of its own a chain of 9,000 observed states needed 298 GB of slabs instead of
+// 248, and one of 1,200 had room for one CTA per SM instead of two.)
 struct SweepSlab {
-  size_t A, af, piv, by, rv, x, xt, z, yp, vec, sf, qp, qf, total;
+  size_t A, piv, by, rv, x, xt, z, yp, vec, sf, qp, qf, total;
 };
 // Entries of a warp's draw buffer: the longest row, in whole warps (none below the register form).
 __host__ __device__ inline size_t draw_ld(int32_t c) { return c + 1 <= 128 ? 0 : ((size_t)c + 32) & ~size_t(31); }
@@ -63,8 +66,6 @@ __host__ __device__ inline SweepSlab sweep_slab(int32_t n, int32_t c) {
   const size_t cc = (size_t)(c > 0 ? c : 1), nn = (size_t)n;
   SweepSlab s{};
   size_t o = 0;
-  s.A = o;   o = up256(o + 8 * cc * cc);
-  s.af = o;  o = up256(o + 4 * cc * cc);
   s.piv = o; o = up256(o + 4 * cc);
   s.by = o;  o = up256(o + 8 * cc);
   s.rv = o;  o = up256(o + 8 * cc);
@@ -76,6 +77,7 @@ __host__ __device__ inline SweepSlab sweep_slab(int32_t n, int32_t c) {
   s.sf = o;  o = up256(o + 4 * nn);
   s.qp = o;  o = up256(o + 8 * cc * (cc + 1));
   s.qf = o;  o = up256(o + 4 * nn * (cc + 1));
+  s.A = o;   o = up256(o + 8 * cc * cc);
   s.total = o;
   return s;
 }
@@ -970,7 +972,6 @@ perturb_kernel(ChainDev C, afc_perturb_params pp, const double *mu0, const doubl
   unsigned char *slab = slabs + (size_t)blockIdx.x * slab_bytes;
   const SweepSlab L = sweep_slab(n, c);
   double *A = reinterpret_cast<double *>(on_chip ? smem : slab + L.A);
-  float *af = reinterpret_cast<float *>(slab + L.af);
   int32_t *piv = reinterpret_cast<int32_t *>(slab + L.piv);
   double *by = reinterpret_cast<double *>(slab + L.by), *rv = reinterpret_cast<double *>(slab + L.rv);
   double *x = reinterpret_cast<double *>(slab + L.x), *z = reinterpret_cast<double *>(slab + L.z);
@@ -1097,6 +1098,7 @@ perturb_kernel(ChainDev C, afc_perturb_params pp, const double *mu0, const doubl
           // blocked LU of an FP32 copy, then FP64 iterative refinement against the FP64 matrix; if
           // the refinement stalls, the FP64 blocked LU of A itself
           const size_t cc = (size_t)c * c;
+          float *af = reinterpret_cast<float *>(qp);   // the C rows are in A by now
           for (size_t k = threadIdx.x; k < cc; k += blockDim.x) af[k] = (float)A[k];
           __syncthreads();
           bool mixed = lu_factor_blocked_t<float>(af, c, c, piv, ls, reinterpret_cast<float *>(tile));

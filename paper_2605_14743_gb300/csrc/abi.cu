@@ -51,6 +51,14 @@ DevInfo dev_info() {
   return d;
 }
 
+cudaError_t allow_shared(const void *kernel, size_t fixed) {
+  int dev = 0, optin = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              std::max(0, optin - (int)fixed));
+}
+
 }  // namespace afc
 
 namespace {

@@ -49,6 +49,12 @@ afc_result *build_result(int32_t n, uint32_t R, const uint32_t *dense, const dou
                          const double *s, const double *f, double tie_rel, void *stream);
 afc_host_query host_query_of(const afc_graph *g, const afc_params *p, uint32_t n_perturb);
 
+// Lets launches of `kernel` take as much dynamic shared memory as the device has beside `fixed` bytes
+// (at least the kernel's static arrays).  The limit belongs to the kernel, not to the launch: where
+// each launch set its own size, one of another host thread could lower it in between, and the launch
+// failed.
+cudaError_t allow_shared(const void *kernel, size_t fixed);
+
 // mc_kernel.cu: the shared-memory path (one warp per source, settle steps)
 // Shared memory of a counting CTA of the shared-memory path: a graph of n nodes and `arcs`
 // arcs, and `nsw` warps that each own one source slot.

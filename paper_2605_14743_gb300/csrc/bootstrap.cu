@@ -198,7 +198,7 @@ cudaError_t launch_bootstrap(const ChainDev &C, const int32_t *rec, uint32_t R, 
   if (grid == 0) return cudaErrorMemoryAllocation;
   const uint32_t dyn = a_smem ? (uint32_t)a_bytes
                               : (uint32_t)(sizeof(double) * lu_blocked_smem_doubles());
-  cudaFuncSetAttribute(bootstrap_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+  allow_shared(reinterpret_cast<const void *>(bootstrap_kernel), 1024);
   bootstrap_kernel<<<(unsigned)grid, kBootThreads, dyn, stream>>>(
       C, rec, R, B, (uint32_t)seed, (uint32_t)(seed >> 32), slabs, slab, a_smem ? 1 : 0, b_rep,
       T_rep, status);

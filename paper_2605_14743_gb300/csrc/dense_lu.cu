@@ -32,6 +32,7 @@ constexpr int kNb = 8;               // columns of a panel
 constexpr int kSingle = 112;         // matrices up to this size are one panel
 constexpr int kPanelThreads = 1024;
 constexpr int kTile = 32;            // rows and columns of an update tile
+constexpr int kPanelStatic = 4096;   // at least the panel kernel's static arrays
 
 // Leading dimension of the panel in shared memory: odd, so that the elements of a row (one per
 // column) fall into different banks when it is filled and written back.
@@ -250,15 +251,14 @@ lu_update_kernel(LuBatch B, int c, int kb, int nb) {
 cudaError_t launch_lu(const LuBatch &B, int32_t c, int32_t count, int smem_optin,
                       cudaStream_t stream) {
   if (c <= 0 || count <= 0) return cudaSuccess;
-  const size_t cap = (size_t)std::max(0, smem_optin - 4096);   // the panel kernel's static arrays
+  const size_t cap = (size_t)std::max(0, smem_optin - kPanelStatic);
   const bool single = c <= kSingle && panel_bytes(c + 1, c + 1) <= cap;
   for (int kb = 0; kb < c;) {
     const int nb = single ? c : std::min(kNb, c - kb), ke = kb + nb;
     const int last = ke >= c ? 1 : 0;
     const size_t bytes = panel_bytes(c - kb + 1, nb + last);
     if (bytes <= cap) {
-      // the attribute is the kernel's limit: set to the most that any launch may take
-      cudaFuncSetAttribute(lu_panel_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap);
+      allow_shared(reinterpret_cast<const void *>(lu_panel_kernel<true>), kPanelStatic);
       lu_panel_kernel<true><<<count, kPanelThreads, bytes, stream>>>(B, c, kb, nb, last);
     } else {
       lu_panel_kernel<false><<<count, kPanelThreads, 0, stream>>>(B, c, kb, nb, last);

@@ -266,9 +266,7 @@ cudaError_t launch_brandes_t(const McDev *Pd, BigGroup *groups, uint32_t ngroups
                              uint32_t smem_bytes, int slots_on_chip, uint32_t grid,
                              cudaStream_t stream) {
   const uint32_t smem = slots_on_chip ? smem_bytes : (uint32_t)sizeof(CtaCtl);
-  if (smem > 48u * 1024u)
-    cudaFuncSetAttribute(big_brandes_kernel<BLOCK, TS>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  allow_shared(reinterpret_cast<const void *>(big_brandes_kernel<BLOCK, TS>), 0);
   big_brandes_kernel<BLOCK, TS><<<grid, BLOCK, smem, stream>>>(
       Pd, groups, ngroups, arena, stride, spt, mode, slots_on_chip);
   return cudaGetLastError();
@@ -284,9 +282,7 @@ cudaError_t launch_steps_t(const McDev *Pd, BigGroup *groups, uint32_t ngroups,
                            unsigned char *arena, size_t stride, uint32_t nsw, int mode,
                            uint32_t smem_bytes, int dist_on_chip, uint32_t grid,
                            cudaStream_t stream) {
-  if (smem_bytes > 48u * 1024u)
-    cudaFuncSetAttribute(big_steps_kernel<BLOCK, LONG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         smem_bytes);
+  allow_shared(reinterpret_cast<const void *>(big_steps_kernel<BLOCK, LONG>), 0);
   big_steps_kernel<BLOCK, LONG><<<grid, BLOCK, smem_bytes, stream>>>(Pd, groups, ngroups, arena, stride,
                                                                nsw, mode, dist_on_chip);
   return cudaGetLastError();

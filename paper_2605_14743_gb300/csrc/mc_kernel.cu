@@ -401,8 +401,7 @@ static cudaError_t launch_counts_t(const McDev *probs_dev, int nprob, uint64_t *
                                    uint64_t total_items, uint32_t nsw, uint32_t smem,
                                    uint32_t grid, unsigned char *scratch, size_t stride,
                                    cudaStream_t stream) {
-  cudaFuncSetAttribute(mc_counts_kernel<BLOCK, LONG, CHIP>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  allow_shared(reinterpret_cast<const void *>(mc_counts_kernel<BLOCK, LONG, CHIP>), 0);
   mc_counts_kernel<BLOCK, LONG, CHIP><<<grid, BLOCK, smem, stream>>>(
       probs_dev, nprob, prefix_dev, total_items, nsw, scratch, stride);
   return cudaGetLastError();
@@ -438,7 +437,7 @@ cudaError_t launch_debug_realize(const McDev &P, uint32_t r_count, uint8_t *aliv
 cudaError_t launch_debug_components(const McDev &P, uint32_t r_count, int32_t *comp, int32_t *csize,
                                     cudaStream_t stream) {
   const uint32_t smem = components_smem_bytes(P.n, (uint32_t)(2 * P.m));
-  cudaFuncSetAttribute(debug_components_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  allow_shared(reinterpret_cast<const void *>(debug_components_kernel), 0);
   debug_components_kernel<<<r_count, 256, smem, stream>>>(P, comp, csize);
   return cudaGetLastError();
 }
@@ -451,7 +450,7 @@ static cudaError_t launch_sssp_t(const McDev &P, uint32_t r, const int32_t *sour
   L.make((uint32_t)P.n, (uint32_t)(2 * P.m), nsw);
   const int32_t nw = (int32_t)L.wide_slots(nsw);
   const uint32_t grid = (uint32_t)((nsrc + nw - 1) / nw);
-  cudaFuncSetAttribute(debug_sssp_kernel<BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  allow_shared(reinterpret_cast<const void *>(debug_sssp_kernel<BLOCK>), 0);
   debug_sssp_kernel<BLOCK><<<grid, BLOCK, smem, stream>>>(P, r, sources, nsrc, nsw, long_form ? 1 : 0,
                                                        dist, sigma);
   return cudaGetLastError();

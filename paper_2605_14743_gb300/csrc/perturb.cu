@@ -38,6 +38,7 @@ constexpr int kThreadsOnChip = 512, kThreadsSlab = 256;
 __host__ __device__ constexpr int sweep_threads(bool on_chip) { return on_chip ? kThreadsOnChip : kThreadsSlab; }
 constexpr int kMaxK2 = 32;
 constexpr int kMaxHist = 64;
+constexpr int kSweepStatic = 8 * 1024;   // at least the sweep kernel's static arrays
 
 // Leading dimension of the FP32 inverse: whole 128-byte lines, padded with zeros.
 __host__ __device__ inline size_t inv_ld(int32_t c) { return ((size_t)(c > 0 ? c : 1) + 31) & ~size_t(31); }
@@ -1342,8 +1343,6 @@ cudaError_t launch_perturb(const ChainDev &C, const afc_perturb_params &pp, cons
   int max_optin = 0, dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  // attributes set on every launch: they are the kernel's limit, and an earlier launch may have
-  // left it below what this one needs
   float *inv = nullptr, *inv_t = nullptr;
   const int nr = inverse_smem(c, 8) <= (size_t)max_optin - 1024 ? 8 : 2;   // c up to 5,900 / 23,700
   if (c > 0 && inverse_smem(c, nr) <= (size_t)max_optin - 1024) {
@@ -1351,7 +1350,7 @@ cudaError_t launch_perturb(const ChainDev &C, const afc_perturb_params &pp, cons
     inv_t = inv + (size_t)c * inv_ld(c);
     cudaMemsetAsync(inv, 0, perturb_inverse_bytes(c), stream);
     auto kernel = nr == 8 ? inverse32_kernel<8> : inverse32_kernel<2>;
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)inverse_smem(c, nr));
+    allow_shared(reinterpret_cast<const void *>(kernel), 1024);
     kernel<<<(c + nr - 1) / nr, kInvThreads, inverse_smem(c, nr), stream>>>(lu0, piv0, c, inv_ld(c),
                                                                            inv, inv_t);
   }
@@ -1363,10 +1362,10 @@ cudaError_t launch_perturb(const ChainDev &C, const afc_perturb_params &pp, cons
   const size_t sums = 8 * (size_t)(threads / 32) * (size_t)(c > 0 ? c : 1);
   const size_t mat = on_chip ? up256(8 * (size_t)(c > 0 ? c : 1) * (size_t)(c > 0 ? c : 1)) : 0;
   const size_t vec = vec_bytes(c, threads) - sums + std::max(sums, tiles);
-  const int vec_smem = mat + vec + 8 * 1024 <= (size_t)max_optin ? 1 : 0;
+  const int vec_smem = mat + vec + kSweepStatic <= (size_t)max_optin ? 1 : 0;
   const size_t dyn = vec_smem ? mat + vec : std::max(mat, tiles);
   auto kernel = on_chip ? perturb_kernel<true> : perturb_kernel<false>;
-  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+  allow_shared(reinterpret_cast<const void *>(kernel), kSweepStatic);
   int per_sm = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, dyn);
   if (e != cudaSuccess) return e;

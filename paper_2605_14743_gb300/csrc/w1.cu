@@ -437,7 +437,7 @@ cudaError_t launch_w1(int32_t n, int64_t m, const int32_t *rp, const int32_t *co
   if (count <= 0) return cudaSuccess;
   const size_t slot = slot_bytes(n, m);
   const int dyn = mode == 2 ? (int)(slot + graph_bytes(n, m)) : mode == 1 ? (int)slot : 0;
-  cudaFuncSetAttribute(w1_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+  allow_shared(reinterpret_cast<const void *>(w1_kernel), 0);
   w1_kernel<<<grid, 32, dyn, stream>>>(n, m, rp, col, eid, x, y, count, out, slab, slot, mode,
                                        status);
   return cudaGetLastError();

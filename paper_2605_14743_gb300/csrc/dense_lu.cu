@@ -23,6 +23,7 @@
 
 #include "afc_internal.h"
 #include "dense_lu.cuh"
+#include "linalg.cuh"
 
 namespace afc {
 
@@ -40,24 +41,6 @@ __host__ __device__ inline int panel_ld(int rows) { return ((rows + 15) & ~15) +
 
 __host__ inline size_t panel_bytes(int rows, int cols) {
   return sizeof(double) * (size_t)panel_ld(rows) * (size_t)cols;
-}
-
-// |x| as an integer that orders like the magnitude; NaN never wins (0).  Integer compares keep the
-// pivot search off the FP64 pipe.
-__device__ __forceinline__ unsigned long long mag(double x) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
-  return b > 0x7FF0000000000000ull ? 0ull : b;
-}
-
-// Largest key over the warp's lanes, ties to the smallest index; every lane gets both.
-__device__ __forceinline__ void warp_argmax(unsigned long long &key, int &idx) {
-  const uint32_t hi = (uint32_t)(key >> 32);
-  const uint32_t mh = __reduce_max_sync(0xFFFFFFFFu, hi);
-  const uint32_t lo = hi == mh ? (uint32_t)key : 0u;
-  const uint32_t ml = __reduce_max_sync(0xFFFFFFFFu, lo);
-  const bool top = hi == mh && (uint32_t)key == ml;
-  idx = (int)__reduce_min_sync(0xFFFFFFFFu, top ? (uint32_t)idx : 0x7FFFFFFFu);
-  key = ((unsigned long long)mh << 32) | ml;
 }
 
 // Panel kb .. kb + nb - 1 of problem blockIdx.x: rows kb .. c - 1 and the extra row; with_col: the

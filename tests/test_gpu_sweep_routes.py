@@ -27,3 +27,18 @@ def test_wide_moves_are_corrected(n, c, lengths, radius):
     assert max_rel(mx, [ref.max_db, ref.max_lin_err, ref.max_rowsum_N]) < 1e-9
     assert (hst == ref.shift_hist).all()
     assert stats.cpu().numpy().tolist() == [P, 0]
+
+
+@pytest.mark.parametrize("c", [1, 2, 31, 32, 33, 97, 160])
+def test_factored_on_chip(c):
+    """The multiplicative model's perturbations are factored in shared memory: pivots at the edges of
+    a warp's rows, with rows that move (few entries, little absorption)."""
+    n, R, P = 170, 6000, 5
+    counts = _counts(n, c, [1, 2, 3, 40], R, c, False)
+    ch = Chain(counts, R, 0.0)
+    Q, r = O.assemble_q(counts, R, 0.0)
+    cnt, pairs, hst, mx, bo = ch.sweep(0, P, 0.9, 0.01, 7, model=1)
+    ref = O.perturb_sweep(Q, r, None, 0, P, 0.9, 0.01, 7, keep=True, model=1)
+    assert close(bo, ref.b)
+    assert max_rel(mx, [ref.max_db, ref.max_lin_err, ref.max_rowsum_N]) < 1e-9
+    assert (hst == ref.shift_hist).all()

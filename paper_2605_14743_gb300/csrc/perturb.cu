@@ -954,7 +954,7 @@ __device__ __forceinline__ void atomic_max_pos(double *addr, double v) {
 }
 
 // ON_CHIP: the factorisation's matrix in shared memory (small c); vec_smem: the vectors there.
-// inv null: always factor (columns too long for the inverse's kernel).
+// inv null: always factor (the shortest chains, and columns too long for the inverse's kernel).
 template <bool ON_CHIP>
 __global__ void __launch_bounds__(sweep_threads(ON_CHIP), kPerturbCtasPerSm)
 perturb_kernel(ChainDev C, afc_perturb_params pp, const double *mu0, const double *b0,
@@ -1032,9 +1032,9 @@ perturb_kernel(ChainDev C, afc_perturb_params pp, const double *mu0, const doubl
   R.radius_f = R.always_general ? 0.0f : trunc_f32(pp.l1_radius);
   R.floor_f = trunc_f32(pp.r_min) * 1.0001f;
   R.screen = R.always_general ? 4e-7f : 1.2e-6f * fminf(R.radius_f, 2.0f) + 4e-7f;
-  // the multiplicative moves of the robust search (50% an entry) rarely contract 5x a round; on chip
-  // the factorisation is the cheaper try for them
-  const bool try_defect = inv != nullptr && !(on_chip && pp.model == 1);
+  // the multiplicative moves of the robust search (50% an entry) and l1 moves of more than three
+  // quarters of a row rarely contract 5x a round; on chip the factorisation is the cheaper try for them
+  const bool try_defect = inv != nullptr && !(on_chip && (pp.model == 1 || pp.l1_radius > 0.75));
   uint32_t loc_defect = 0, loc_factored = 0;
   const uint32_t p_end = pp.p_begin + pp.p_count;
   for (uint32_t p = pp.p_begin + blockIdx.x; p < p_end; p += gridDim.x) {
@@ -1358,7 +1358,12 @@ cudaError_t launch_perturb(const ChainDev &C, const afc_perturb_params &pp, cons
   cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   float *inv = nullptr, *inv_t = nullptr;
   const int nr = inverse_smem(c, 8) <= (size_t)max_optin - 1024 ? 8 : 2;   // c up to 5,900 / 23,700
-  if (c > 0 && inverse_smem(c, nr) <= (size_t)max_optin - 1024) {
+  // The shortest chains are factored: the factorisation costs less than the rounds of the
+  // corrections and the inverse before them, with wide moves (more rounds) up to a larger size.
+  // Factored / corrected, us a call: radius 0.05, 304 perturbations c = 8 134 / 218, 16 189 / 265, 24
+  // 301 / 340, 32 346 / 349, one perturbation c = 24 249 / 242, 32 291 / 251; radius 0.5 c = 32 375 / 490.
+  const int32_t direct = pp.model == 0 && pp.l1_radius > 0.3 ? 40 : 24;
+  if (c > direct && inverse_smem(c, nr) <= (size_t)max_optin - 1024) {
     inv = reinterpret_cast<float *>(ws + L.off_inv);
     inv_t = inv + (size_t)c * inv_ld(c);
     cudaMemsetAsync(inv, 0, perturb_inverse_bytes(c), stream);

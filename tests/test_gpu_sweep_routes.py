@@ -42,3 +42,19 @@ def test_factored_on_chip(c):
     assert close(bo, ref.b)
     assert max_rel(mx, [ref.max_db, ref.max_lin_err, ref.max_rowsum_N]) < 1e-9
     assert (hst == ref.shift_hist).all()
+
+
+@pytest.mark.parametrize("c", [24, 25, 40, 41])
+@pytest.mark.parametrize("radius", [0.05, 0.29, 0.31, 0.8])
+def test_short_chains(c, radius):
+    """Around the sizes and widths up to which a chain is factored without corrections."""
+    n, R, P = 90, 6000, 5
+    counts = _counts(n, c, [2, 9, c], R, c, False)
+    ch = Chain(counts, R, 0.15)
+    Q, r = O.assemble_q(counts, R, 0.15)
+    cnt, pairs, hst, mx, bo = ch.sweep(0, P, radius, 0.05, 7)
+    ref = O.perturb_sweep(Q, r, None, 0, P, radius, 0.05, 7, keep=True)
+    assert close(bo, ref.b, rel=1e-12)
+    assert max_rel(mx, [ref.max_db, ref.max_lin_err, ref.max_rowsum_N]) < 1e-9
+    assert cnt.tolist() == [ref.top1_changes, ref.topk_set_changes, ref.topk_order_changes]
+    assert (pairs == ref.pair_flips).all() and (hst == ref.shift_hist).all()

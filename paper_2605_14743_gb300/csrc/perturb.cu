@@ -860,22 +860,17 @@ __device__ __forceinline__ void correct(const SweepCtx &X, double *x, float m[2]
 // 5x has come down to the defects' rounding (below 1e-15: converged too) or stalls.  The rounding
 // grows with the change: at l1 moves of 0.5 it is reached before 1e-17, and without that rule every
 // such perturbation was factored (c = 200, 304 perturbations: 4.9 ms a call, 1.66 with it; c = 1,900,
-// 32: 285 and 28 ms).  A call in the slab kernel, whose loops become 10% slower with these few lines
-// inlined (c = 914); inlined on chip, where the call costs 0.7%.
+// 32: 285 and 28 ms).  In FP32, like the corrections themselves: every thread keeps the account, and
+// in FP64 it took 3% of a sweep's time at c = 97 (4.88 -> 4.72 ms, 2,000 perturbations) and 10% at
+// c = 914.  The scale is finite, so an infinite or NaN correction never converges.
 struct Progress {
-  double scale, prev = 0.0;
+  float scale, prev = 0.0f;
   bool done = false, stalled = false;
-  template <int THREADS>
-  __device__ __forceinline__ void step(int it, double dm) {
-    if constexpr (THREADS == kThreadsSlab) call(it, dm);
-    else rule(it, dm);
-  }
-  __device__ __noinline__ void call(int it, double dm) { rule(it, dm); }
-  __device__ __forceinline__ void rule(int it, double dm) {
+  __device__ __forceinline__ void step(int it, float dm) {
     if (done) return;
-    if (dm <= 1e-17 * scale || (it > 0 && dm < 0.2 * prev && dm * dm <= 1e-17 * scale * prev)) done = true;
-    else if (it >= 2 && !(dm < 0.2 * prev)) {
-      done = dm <= 1e-15 * scale;
+    if (dm <= 1e-17f * scale || (it > 0 && dm < 0.2f * prev && dm * dm <= 1e-17f * scale * prev)) done = true;
+    else if (it >= 2 && !(dm < 0.2f * prev)) {
+      done = dm <= 1e-15f * scale;
       stalled = !done;
     }
     prev = dm;
@@ -892,7 +887,7 @@ struct Progress {
 // is zero before and after.
 template <int THREADS>
 __device__ inline bool defect_solve(const SweepCtx &X, const double *mu0, const double *t0,
-                                    double mu_scale, double t_scale) {
+                                    float mu_scale, float t_scale) {
   for (int32_t k = threadIdx.x; k < X.c; k += THREADS) {
     X.mu[k] = 0.0;
     X.t[k] = 0.0;
@@ -904,8 +899,8 @@ __device__ inline bool defect_solve(const SweepCtx &X, const double *mu0, const 
   for (int it = 0; it < 40; ++it) {
     float m[2];
     correct<THREADS, true>(X, X.mu, m);
-    pm.step<THREADS>(it, (double)m[0]);
-    pt.step<THREADS>(it, (double)m[1]);
+    pm.step(it, m[0]);
+    pt.step(it, m[1]);
     if (pm.done && pt.done) {
       for (int32_t k = threadIdx.x; k < X.c; k += THREADS) {
         X.mu[k] += mu0[X.c_list[k]];
@@ -927,7 +922,7 @@ __device__ inline bool defect_solve(const SweepCtx &X, const double *mu0, const 
 // z (I - Q_CC) = x on the nominal rows (the first-order prediction), to 1e-17 of scale; rm is
 // overwritten.  Two to three rounds: only the inverse's rounding is corrected.
 template <int THREADS>
-__device__ inline bool nominal_solve(const SweepCtx &X, double *z, double scale) {
+__device__ inline bool nominal_solve(const SweepCtx &X, double *z, float scale) {
   for (int32_t k = threadIdx.x; k < X.c; k += THREADS) {
     z[k] = 0.0;
     X.rm[k] = trunc_f32(X.x[k]);
@@ -937,7 +932,7 @@ __device__ inline bool nominal_solve(const SweepCtx &X, double *z, double scale)
   for (int it = 0; it < 12; ++it) {
     float m[2];
     correct<THREADS, false>(X, z, m);
-    pz.step<THREADS>(it, (double)m[0]);
+    pz.step(it, m[0]);
     if (pz.done) return true;
     if (pz.stalled) return false;
     defect_rows<THREADS, true>(X, z);
@@ -1022,10 +1017,10 @@ perturb_kernel(ChainDev C, afc_perturb_params pp, const double *mu0, const doubl
   for (int32_t i = threadIdx.x; i < n; i += blockDim.x) { part += mu0[i]; pmx = fmax(pmx, mu0[i]); }
   const double T0 = block_sum(part, red);
   const double invT0 = 1.0 / T0;
-  const double mu0_max = block_max(pmx, red);
+  const float mu0_max = fminf((float)block_max(pmx, red), 1e30f);   // finite: see Progress
   pmx = 0.0;
   for (int32_t k = threadIdx.x; k < c; k += blockDim.x) pmx = fmax(pmx, t0[k]);
-  const double t0_max = block_max(pmx, red);
+  const float t0_max = fminf((float)block_max(pmx, red), 1e30f);
   double loc_db = 0.0, loc_lin = 0.0, loc_t = 0.0;
   RowArgs R{nzcol, C.c_list, nzval, c, (uint32_t)n, 0u, (uint32_t)pp.seed, (uint32_t)(pp.seed >> 32),
             pp.model, pp.l1_radius, pp.r_min, pp.rel_radius, 0.0f, 0.0f, 0.0f, !(pp.l1_radius <= 1e6)};

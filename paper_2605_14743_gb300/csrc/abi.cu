@@ -241,8 +241,13 @@ McPlan plan_for(const afc_mc_problem &p0, uint32_t nmax, uint64_t amax, uint64_t
   if (p0.block_threads) {
     pl.block = p0.block_threads;
   } else if (pl.chip) {
+    // With FP32 and recheck, realizations that are done again in FP64 take twice as long and the call
+    // waits for the last ones: from 128 nodes twice as many realizations before a step down (R = 600,
+    // n = 140 / 200 / 240: 1.63 / 2.76 / 3.05 -> 1.46 / 2.41 / 2.99 ms; n = 60 0.53 -> 0.58).
     const uint64_t warps = (uint64_t)std::max(1, d.sms) * (kSmallThreadsPerSm / 32);
-    pl.block = total_items * 8u >= warps ? 256 : total_items * 16u >= warps ? 512 : 1024;
+    const uint64_t items =
+        p0.precision == AFC_FP32_RECHECK && nmax >= 128 ? total_items / 2 : total_items;
+    pl.block = items * 8u >= warps ? 256 : items * 16u >= warps ? 512 : 1024;
   } else {
     // the smallest CTA that holds a warp for every slot that fits (fewer threads per CTA leave
     // each thread more registers for the source warps' caches)

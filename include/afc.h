@@ -340,7 +340,8 @@ int afc_bootstrap(const afc_chain *chain, const int32_t *next_states, const int3
  * v_j - v_bot first, ties by j).  DEVICE in: counts [n][n+1], v [n].  DEVICE out: T [n],
  * Qstar [n][n] a minimising kernel (or NULL).  Workspace: 256 bytes (T holds the columns' order
  * while the rows are solved: T and v do not overlap).  SYNCHRONISES `stream`.
- * Errors: AFC_EINVAL when some U_i is empty (its lower bounds exceed 1 - r_min). */
+ * Errors: AFC_EINVAL when some U_i is empty (its lower bounds exceed 1 - r_min), AFC_EDEVICE when
+ * the launch's CTAs do not meet (its barriers give up after about a second). */
 int afc_robust_inner(const afc_chain *chain, const uint32_t *counts, double eps, double r_min,
                      int32_t support_only, const double *v, double v_bot, double *T, double *Qstar,
                      void *workspace, size_t workspace_bytes, void *stream);
@@ -351,8 +352,8 @@ int afc_robust_inner(const afc_chain *chain, const uint32_t *counts, double eps,
  * minimises, +1 maximises.  Policy iteration: the inner problem's optimiser at V, V of that
  * kernel by an FP64 LU of I - Q*, until V changes by at most 1e-13 relative (at most 100
  * rounds).  DEVICE out: V [n], Qstar [n][n] (or NULL), b_star [n] = the AFC of P*, scalars [2]
- * = {E_s[T] under P*, b* . f}; HOST out: *iterations (or NULL).  n <= 4096 (dense solve in one
- * CTA).  Workspace: afc_robust_value_workspace(n).  SYNCHRONISES `stream`.  Errors as
+ * = {E_s[T] under P*, b* . f}; HOST out: *iterations (or NULL).  n <= 4096 (dense solves
+ * over the whole GPU).  Workspace: afc_robust_value_workspace(n).  SYNCHRONISES `stream`.  Errors as
  * afc_robust_inner, AFC_ESINGULAR for a zero pivot. */
 size_t afc_robust_value_workspace(int32_t n);
 int afc_robust_value(const afc_chain *chain, const uint32_t *counts, double eps, double r_min,
@@ -368,8 +369,8 @@ int afc_robust_value(const afc_chain *chain, const uint32_t *counts, double eps,
  * a robust value that policy iteration computes exactly on a rectangular set (afc_robust_value
  * with that reward); Dinkelbach's iteration lambda <- b_v(argopt) from lambda = 0 reaches the
  * root (until lambda moves by at most 1e-13 relative, at most 60 steps).  The 2k problems (the
- * supremum and the infimum for each of the k HOST nodes) run as one batch: one CTA each for the
- * dense FP64 LU of I - Q*.  HOST out: b_lo [k], b_hi [k], iterations [2k] (or NULL: Dinkelbach
+ * supremum and the infimum for each of the k HOST nodes) run as one batch, their dense
+ * FP64 LUs of I - Q* together over the whole GPU.  HOST out: b_lo [k], b_hi [k], iterations [2k] (or NULL: Dinkelbach
  * steps of the supremum, then the infimum, per node).  n <= 4096.  Workspace:
  * afc_robust_envelope_workspace(n, k) (2 n^2 + O(n) doubles per problem).  SYNCHRONISES
  * `stream`.  Errors as afc_robust_value; AFC_EDEVICE when Dinkelbach does not settle. */

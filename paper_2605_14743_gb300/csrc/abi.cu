@@ -77,8 +77,7 @@ uint32_t auto_delta(const afc_mc_problem &p) {
 }
 
 int auto_block(const afc_mc_problem &p) {
-  // measured: 1024-thread CTAs with one-warp teams are the fastest shape for small graphs too
-  // (n = 64: 1.7x the former 256-thread CTAs)
+  // 1024: the global path's CTA; on the shared path plan_for chooses by what fits
   return p.block_threads ? p.block_threads : 1024;
 }
 
@@ -268,9 +267,9 @@ McPlan plan_for(const afc_mc_problem &p0, uint32_t nmax, uint64_t amax, uint64_t
   return pl;
 }
 
-// The global path's settle-step kernel when shared memory holds the distance arrays of at
-// least this many warps (about 14,000 nodes) and steps_beat_buckets; otherwise the bucketed
-// kernel.
+// The global path's settle-step kernel when steps_beat_buckets and shared memory holds the distance
+// arrays of at least this many warps (a guard: at that rule's 7,200 nodes 227 KB hold 7); otherwise
+// the bucketed kernel.
 constexpr uint32_t kMinStepWarps = 4;
 
 // Whether the settle-step kernel outruns the bucketed one on this graph.  Its cost grows with
@@ -283,9 +282,13 @@ constexpr uint32_t kMinStepWarps = 4;
 // 0.94, 1000 1.04 / 0.82; n = 5,000: W = 10 1.39 / 1.24, 50 1.13 / 1.01, 100 0.93 / 0.76; n =
 // 6,007: W = 50 1.06 / 0.93, 100 0.82 / 0.69; n = 8,000: W = 10 0.88 / 0.77, 25 0.94 / 0.80; n =
 // 10,500: W = 1 0.68 / 0.62, 10 0.63 / 0.55; n = 12,000: W = 10 0.54 / 0.47; at n = 6,600, W = 10
-// 1.04 / 0.91, and 1.10 on WS k = 10.  So: at most 7,200 nodes whatever the lengths, and n min(W, 200)^0.35 <= 19,500, the crossover of the ER graphs
-// (n = 5,000 for W = 50, 3,900 for W = 100, 3,050 for W >= 200).  Per-edge length ranges and
-// length laws count as W = 65,535.
+// 1.04 / 0.91, and 1.10 on WS k = 10.  So: at most 7,200 nodes whatever the lengths, and
+// n min(W, 200)^0.35 <= 19,500 (n = 5,000 for W = 50, 3,900 for W = 100, 3,050 for W >= 200), about
+// the crossover of the ER graphs for W = 50 and 100.  The line is older than the LONG form, which
+// flattened the dependence on W: by the ratios above it sends graphs to the buckets that the settle
+// steps would run faster (n = 3,200, W = 1000: 31% on WS, 6% on ER; n = 5,000, W = 50: 13% and 1%)
+// and keeps ER graphs of 6,600 nodes with W = 10 that lose 9%.  Per-edge length ranges and length
+// laws count as W = 65,535.
 bool steps_beat_buckets(const afc_mc_problem &p) {
   const double w = (p.w_hi || p.wtab_ptr) ? 65535.0 : (double)std::max<uint32_t>(p.w_hi_all, 1u);
   return p.n <= 7200 && (double)p.n * std::pow(std::min(w, 200.0), 0.35) <= 19500.0;

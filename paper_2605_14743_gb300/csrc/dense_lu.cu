@@ -13,10 +13,12 @@
 // multipliers are z = y U^-1.  A column vector b (solving A x = b) rides along as a column right of
 // it and becomes L^-1 P b.  One triangular solve each is left (upper_solve, lower_t_solve).
 //
-// Bound: GB300's FP64 pipe (about 2 FMA per clock and SM).  The trailing updates take c^3 / 3 FMA
-// over all SMs, the panels c^2 kNb / 4 on one SM and about 0.4 us of latency per column, the
-// launches about 7 us per panel, hence kNb = 8 (at c = 1,251: 1.1 + 0.7 + 0.5 + 1.0 ms).  Before,
-// one CTA eliminated column by column: 222 ms at c = 1,251, 0.80 ms at c = 97.
+// Bound: the chain panel, rows, update of every kNb columns.  By GB300's FP64 pipe (about 2 FMA per
+// clock and SM) the trailing updates' c^3 / 3 FMA take 1.1 ms over all SMs at c = 1,251 and the panels'
+// c^2 kNb / 4 take 0.7 on one SM; the kernels' durations there (profiles/solve_launches.md) are
+// panels 3.7 ms (23 us each, 35 the tallest: pivots and barriers of one CTA), updates 2.0 (13 us), rows
+// 1.0 (6.4 us) and the two triangular solves 0.4, of a call's 7.55.  Before, one CTA eliminated
+// column by column: 222 ms at c = 1,251, 0.80 ms at c = 97.
 #include <algorithm>
 #include <cstdint>
 #include <cuda_runtime.h>

@@ -3,12 +3,12 @@
 // One CTA owns one network realization at a time (persistent over realizations) and keeps
 // it in shared memory:
 //   A1  Philox4x32-10 edge draws -> alive-compacted CSR with packed (neighbour, length) arcs,
-//       and the smallest alive length at every node
+//       and the bounds of the settle steps at every node (its smallest alive lengths)
 //   A2  components by lock-free union-find (root = smallest id), sizes, candidate flags
 //   A3  one warp per source: Dijkstra by settle steps (mc_steps.cuh), source slots on chip
 //   A4  path counts sigma (exact 64-bit) pulled from the settled predecessors in the same arc
 //       scan that relaxes the step's outgoing arcs: one scan per arc in the forward direction
-//   A5  dependencies delta step by step in reverse, one scan per arc; betweenness accumulated
+//   A5  dependencies delta by levels or settle steps in reverse, one scan per arc; betweenness accumulated
 //       exactly in 128-bit fixed point
 //   A6  tie-ruled argmax per valid component (Sec. 3.2 eq. local-center, Sec. 7.1 Sel_W)
 //       and the transition-count update of every anchor (Alg. 1 / Alg. 2)

@@ -13,11 +13,11 @@
 // What bounds it: GB300's FP64 pipe takes 16 cycles per warp instruction and SM (2 lanes a clock),
 // 64 times an FP32 or integer one.  So FP64 is kept for what reaches a result and the rest runs in
 // integers or FP32: a draw's shift is an exact 64-bit integer turned into a double by integer
-// instructions, whether anything clips is decided in FP32 with a margin, and an unclipped entry
-// costs one FP64 multiply-add.  The rows' (N' 1)_i are screened in FP32; the ones that can be the
+// instructions, whether anything clips or reaches the floor is decided in FP32 with a margin (inside it
+// in FP64), and an unclipped entry costs one FP64 multiply-add.  The rows' (N' 1)_i are screened in FP32; the ones that can be the
 // maximum are computed in FP64.  Measured, before (8 FP64 operations per entry, a factorisation or
 // two chains of triangular solves per round, (N' 1) by a thread per row) and now: c = 97, n = 1,000,
-// 2,000 perturbations 13.4 -> 4.8 ms; c = 751, n = 3,000, 304 perturbations 30.8 -> 8.2 ms, its
+// 2,000 perturbations 13.4 -> 4.7 ms; c = 751, n = 3,000, 304 perturbations 30.8 -> 8.2 ms, its
 // kernel with the FP64 pipe 47% and issue 31% active (16 warps per SM wait for loads and chains).
 #include <algorithm>
 #include <cstdint>
@@ -30,7 +30,7 @@
 namespace afc {
 
 // Two resident CTAs per SM: one perturbation's solves are barrier-bound, so two overlap their waits.
-// 512 threads where the matrix fits shared memory (c up to 160: the rows' chains of dependent loads
+// 512 threads where the matrix fits shared memory (c up to 162: the rows' chains of dependent loads
 // and reductions want warps; 64 registers), 256 beyond (every warp has its own column sums, and the
 // blocked factorisation's tiles want 256).
 constexpr int kPerturbCtasPerSm = 2;

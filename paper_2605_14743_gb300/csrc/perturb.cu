@@ -1354,10 +1354,11 @@ cudaError_t launch_perturb(const ChainDev &C, const afc_perturb_params &pp, cons
   float *inv = nullptr, *inv_t = nullptr;
   const int nr = inverse_smem(c, 8) <= (size_t)max_optin - 1024 ? 8 : 2;   // c up to 5,900 / 23,700
   // The shortest chains are factored: the factorisation costs less than the rounds of the
-  // corrections and the inverse before them, with wide moves (more rounds) up to a larger size.
-  // Factored / corrected, us a call: radius 0.05, 304 perturbations c = 8 134 / 218, 16 189 / 265, 24
-  // 301 / 340, 32 346 / 349, one perturbation c = 24 249 / 242, 32 291 / 251; radius 0.5 c = 32 375 / 490.
-  const int32_t direct = pp.model == 0 && pp.l1_radius > 0.3 ? 40 : 24;
+  // corrections and the inverse before them, with wider moves (more rounds) up to a larger size.
+  // Factored / corrected, us for 304 perturbations: radius 0.05 c = 8 134 / 218, 16 189 / 265, 20 244 /
+  // 262; 0.25 c = 20 265 / 335; 0.5 c = 24 337 / 465.  Where both take about the same time the
+  // corrections stay: their results are closer to 64 bits (error 4.3e-16 against 5.3e-16 at c = 16).
+  const int32_t direct = pp.model == 0 && pp.l1_radius > 0.1 ? 24 : 16;
   if (c > direct && inverse_smem(c, nr) <= (size_t)max_optin - 1024) {
     inv = reinterpret_cast<float *>(ws + L.off_inv);
     inv_t = inv + (size_t)c * inv_ld(c);

@@ -44,8 +44,8 @@ def test_factored_on_chip(c):
     assert (hst == ref.shift_hist).all()
 
 
-@pytest.mark.parametrize("c", [24, 25, 40, 41])
-@pytest.mark.parametrize("radius", [0.05, 0.29, 0.31, 0.8])
+@pytest.mark.parametrize("c", [16, 17, 24, 25, 41])
+@pytest.mark.parametrize("radius", [0.05, 0.09, 0.11, 0.5, 0.8])
 def test_short_chains(c, radius):
     """Around the sizes and widths up to which a chain is factored without corrections."""
     n, R, P = 90, 6000, 5
